@@ -144,7 +144,8 @@ typedef struct {
     uint64_t visits;        /* (partition, query) buffers processed; group engine: (partition,
                                group) items and hub chunks */
     uint64_t edges;         /* arcs scanned by the relax/push kernels, counted per query (a
-                               group engine arc counts once per lane it relaxes) */
+                               group engine arc counts once per lane it relaxes; arcs that the
+                               graph leaves out of SSSP are not scanned) */
     uint64_t ops;           /* operations buffered; group engine: target values lowered */
     uint64_t spills;        /* expansions deferred because the op arena was full */
     uint64_t yields;        /* visits that left work behind (yield or budget) */
@@ -182,6 +183,10 @@ void fg_default_graph_opts(fg_graph_opts *o);
  * arrays are copied; the caller keeps ownership. Requires 1 <= n < 2^31 and
  * m < 2^32. Partitions the vertices (Def. 2.1) and stores the graph
  * partition-major on the device. Synchronous. *out receives the handle.
+ * A weighted graph of at least 65,536 arcs, more than half of them between
+ * partitions, also gets a second copy without the arcs that lie on no shortest
+ * path, if enough are found: SSSP in the group engine runs on that copy, with
+ * the same distances (16 * n words of device memory during the call).
  */
 fg_status fg_graph_create(int64_t n, int64_t m, const int64_t *row_ptr, const int32_t *col,
                           const int32_t *w, uint32_t flags, fg_graph **out);

@@ -128,6 +128,24 @@ __device__ __forceinline__ uint32_t g_relax(Ctrl *c, uint32_t d, uint32_t w) {
   return (uint32_t)s;
 }
 
+// Values at or above this can reach 2^32 - 1 when an arc's weight is added.
+__host__ __device__ __forceinline__ uint32_t overflow_limit(const DevGraph &g) {
+  return g.max_w >= kInf - 1u ? 0u : kInf - 1u - g.max_w;
+}
+
+// A vertex's final value on a graph that SSSP runs on without its arcs that
+// lie on no shortest path: reports the overflow that one of the vertex's arcs,
+// left out or not, makes (the relaxations see only the arcs that are in).
+__device__ __forceinline__ void check_all_arcs(const GroupArgs &a, uint32_t lim, uint32_t v, uint32_t d) {
+  if (d == kInf || d < lim) return;
+  const uint32_t e1 = a.all_rp[v + 1];
+  for (uint32_t e = a.all_rp[v]; e < e1; ++e)
+    if ((uint64_t)d + (uint64_t)a.all_wt[e] >= (uint64_t)kInf) {
+      atomicCAS(&a.ctrl->status, 0, (int)FG_ERR_OVERFLOW);
+      return;
+    }
+}
+
 __host__ __device__ constexpr int ilog2c(int x) { return x <= 1 ? 0 : 1 + ilog2c(x / 2); }
 
 // One step of up to 32 arcs, staged by the warp in sarc[0..32): target, weight,
@@ -306,7 +324,7 @@ __global__ void __launch_bounds__(kGThreads, 3) group_kernel(GroupArgs a) {
   const uint64_t tid = (uint64_t)blockIdx.x * kGThreads + threadIdx.x, nthr = (uint64_t)gridDim.x * kGThreads;
   const size_t row = (size_t)a.npad;  // vertices per group row
   // values at or above ovf_lim can overflow when a weight is added
-  const uint32_t ovf_lim = G.max_w >= kInf - 1u ? 0u : kInf - 1u - G.max_w;
+  const uint32_t ovf_lim = overflow_limit(G);
 
   // ---- K0: state and masks (InitBuffers, first half); in serve mode only on
   //      the first launch on the state (later launches resume it) ----
@@ -419,7 +437,9 @@ __global__ void __launch_bounds__(kGThreads, 3) group_kernel(GroupArgs a) {
             const int gg = __ffs(bits) - 1;
             bits &= bits - 1u;
             uint32_t *pv = Dg + (v << LG) + (uint64_t)gg;
-            a.res[((uint64_t)grp * (uint64_t)Gq + (uint64_t)gg) * (uint64_t)G.n + o] = __ldcg(pv);
+            const uint32_t x = __ldcg(pv);
+            a.res[((uint64_t)grp * (uint64_t)Gq + (uint64_t)gg) * (uint64_t)G.n + o] = x;
+            if (QT == Q_SSSP && a.all_rp != nullptr) check_all_arcs(a, ovf_lim, (uint32_t)v, x);
             *pv = kInf;  // the lane starts over for its next request
           }
         }
@@ -1018,24 +1038,29 @@ done:
 // D[group][v][g] (internal order) -> out[row(group * G + g)][orig(v)] for v < n,
 // row(j) = rowmap[j] (or j without a map). A block moves 32 vertices of one
 // group: 32 * G words read as whole lines, transposed in shared memory,
-// written as G runs of 32 values.
-__global__ void __launch_bounds__(256) group_out_kernel(const uint32_t *D, uint32_t *out, const int32_t *orig,
-                                                        const int32_t *rowmap, int64_t n, int64_t npad, int32_t G,
-                                                        int32_t glog2, int32_t nq, int64_t tiles_per_group) {
+// written as G runs of 32 values. Where arcs were left out, the values are
+// held against the overflow limit on the way.
+__global__ void __launch_bounds__(256) group_out_kernel(GroupArgs a, uint32_t *out, const int32_t *rowmap,
+                                                        int64_t tiles_per_group) {
   __shared__ uint32_t t[64][33];
+  const int32_t G = a.G;
+  const int64_t n = a.g.n;
   const int64_t grp = blockIdx.x / tiles_per_group;
   const int64_t v0 = (blockIdx.x % tiles_per_group) * 32;
-  const uint32_t *src = D + ((size_t)grp * (size_t)npad + (size_t)v0) * (size_t)G;
+  const uint32_t lim = overflow_limit(a.g);
+  const uint32_t *src = a.D + ((size_t)grp * (size_t)a.npad + (size_t)v0) * (size_t)G;
   for (int i = threadIdx.x; i < 32 * G; i += blockDim.x) {
-    const int vl = i >> glog2, gq = i & (G - 1);
-    t[gq][vl] = (v0 + vl < n) ? src[i] : kInf;
+    const int vl = i >> a.glog2, gq = i & (G - 1);
+    const uint32_t x = v0 + vl < n ? src[i] : kInf;
+    t[gq][vl] = x;
+    if (a.all_rp != nullptr) check_all_arcs(a, lim, (uint32_t)(v0 + vl), x);
   }
   __syncthreads();
   for (int i = threadIdx.x; i < 32 * G; i += blockDim.x) {
     const int gq = i >> 5, vl = i & 31;
     const int64_t q = grp * G + gq, v = v0 + vl;
-    if (q < nq && v < n) {
-      const int64_t o = orig ? (int64_t)orig[v] : v;
+    if (q < a.nq && v < n) {
+      const int64_t o = a.g.orig ? (int64_t)a.g.orig[v] : v;
       const int64_t r = rowmap ? (int64_t)rowmap[q] : q;
       out[r * n + o] = t[gq][vl];
     }
@@ -1149,7 +1174,7 @@ cudaError_t launch_group_out(const GroupArgs &a, uint32_t *out, const int32_t *r
   const int64_t tiles = (n + 31) / 32;
   const int64_t grid = tiles * (int64_t)a.ngroups;
   if (grid <= 0) return cudaSuccess;
-  group_out_kernel<<<(unsigned)grid, 256, 0, s>>>(a.D, out, a.g.orig, rowmap, n, a.npad, a.G, a.glog2, a.nq, tiles);
+  group_out_kernel<<<(unsigned)grid, 256, 0, s>>>(a, out, rowmap, tiles);
   return cudaGetLastError();
 }
 

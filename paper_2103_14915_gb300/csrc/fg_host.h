@@ -142,6 +142,7 @@ struct fg_graph {
   int engine_qtype = -1;
   uint32_t max_degree = 0;
   double mean_weight = 1.0;        // mean arc weight (1 when unweighted)
+  uint32_t min_weight = 0;         // smallest arc weight (0 when unweighted)
   uint32_t max_weight = 0;         // largest arc weight (0 when unweighted)
   // choices of fg_tune_opts[_ex], keyed by (query kind, log2 of the batch size
   // rounded up, and for PPR the bits of alpha and eps)
@@ -153,6 +154,12 @@ struct fg_graph {
   fg::DevBuf hubs;
   int32_t nhubs = 0;
   uint64_t hub_chunks = 0;
+  // SSSP in the group engine: the graph without the arcs that lie on no
+  // shortest path (fg_reduce.cu), when enough of them were found at creation
+  fg::DevBuf s_rp, s_adj, s_wt, s_hubs;
+  fg::DevGraph s_dg;
+  int32_t s_nhubs = 0;
+  bool reduced = false;
   int group_blocks[4] = {0, 0, 0, 0}, group_threads[4] = {0, 0, 0, 0};
   size_t group_smem[4] = {0, 0, 0, 0};
 };
@@ -168,6 +175,9 @@ constexpr uint32_t kHubChunk = 4096;  // group engine: arcs per hub chunk
 // 8, 16, 32, 64 that holds a smaller batch, and one that fits shared memory);
 // else 1.
 int auto_group_size(const fg_graph *g, int qtype, int64_t nq, bool windowed);
+
+// The graph and hubs a group-engine launch of this query kind runs on.
+void set_group_graph(const fg_graph *g, int qtype, GroupArgs &a);
 
 // One batch of nq queries on workspace ws (see fg_runtime.cpp).
 fg_status run_batch_on(fg_graph *g, Workspace &ws, bool shared_ws, int grid_div, int qtype, const int32_t *src_in,

@@ -144,6 +144,9 @@ struct GroupArgs {
   uint32_t *occ = nullptr;        // [ngroups] lanes holding an admitted, unfinished query
   uint32_t *seen = nullptr;       // [slots] sequence number of each slot's current request
   uint32_t *gact = nullptr;       // [2][ngroups] lanes with pending work in the round of that parity
+  // SSSP on a graph without its arcs that lie on no shortest path (g is then
+  // that graph): the whole graph's arcs, for the overflow test alone
+  const uint32_t *all_rp = nullptr, *all_wt = nullptr;
   uint32_t check_staging = 0;     // 1: compare every staged word with global memory (self-test)
   uint32_t init = 0;              // 1: first launch on this state: fill it before the first round
   uint32_t round0 = 0;            // number of the first round (its parity selects the mask halves)
@@ -190,6 +193,15 @@ cudaError_t launch_group_order(const DevGraph &g, const int32_t *src, int32_t nq
 // Writes the launch's rows to out: slot j's row to out[rowmap[j] * n], or to
 // out[j * n] when rowmap is null.
 cudaError_t launch_group_out(const GroupArgs &a, uint32_t *out, const int32_t *rowmap, cudaStream_t s);
+// Marks the arcs that may lie on a shortest path (fg_reduce.cu): bit e of bits
+// (2 * ceil(m / 64) words) = arc e stays. table: 16 * n words, flags:
+// kReduceRounds + 1 words of scratch. Needs weights and m > 0.
+constexpr int kReduceHubs = 8, kReduceRounds = 16;
+struct HubSet {
+  uint32_t v[kReduceHubs];  // internal ids
+};
+cudaError_t mark_useful_arcs(const DevGraph &g, const HubSet &hubs, uint32_t *table, unsigned *flags, uint32_t *bits,
+                             cudaStream_t s);
 cudaError_t launch_plain(const PlainArgs &a, int blocks, int threads, cudaStream_t s);
 
 // runtime services for entry points outside fg_runtime.cpp

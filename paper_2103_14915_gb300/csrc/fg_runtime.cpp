@@ -134,6 +134,121 @@ static fg_status validate_csr(int64_t n, int64_t m, const int64_t *row_ptr, cons
   return FG_OK;
 }
 
+static void release_reduced(fg_graph *g) {
+  g->s_rp.release(); g->s_adj.release(); g->s_wt.release(); g->s_hubs.release();
+  g->reduced = false;
+}
+
+// The graph that SSSP runs on in the group engine: without the arcs that
+// fg_reduce.cu shows to lie on no shortest path. Built where the group engine
+// is the automatic choice and an arc can be beaten at all (a walk of two arcs
+// is at least twice the smallest weight), for graphs of at least kReduceMinArcs
+// arcs, and kept when it leaves at most 3/4 of them. Without memory for it the
+// graph does without. Other CUDA errors are returned.
+constexpr int64_t kReduceMinArcs = 1 << 16;
+
+static cudaError_t build_reduced(fg_graph *g, const std::vector<uint32_t> &rp, const std::vector<uint32_t> &adj,
+                                 const std::vector<uint32_t> &wt) {
+  const int64_t n = g->n, m = g->m;
+  if (m < kReduceMinArcs || 2 * g->cut <= m) return cudaSuccess;
+  if (2 * (uint64_t)g->min_weight >= (uint64_t)g->max_weight) return cudaSuccess;
+  // the vertices of largest out-degree, ties by smaller id
+  HubSet hubs;
+  uint32_t hdeg[kReduceHubs];
+  int nh = 0;
+  for (int64_t v = 0; v < n; ++v) {
+    const uint32_t deg = rp[(size_t)v + 1] - rp[(size_t)v];
+    if (nh == kReduceHubs && deg <= hdeg[nh - 1]) continue;
+    int k = nh < kReduceHubs ? nh++ : nh - 1;
+    for (; k > 0 && hdeg[k - 1] < deg; --k) {
+      hdeg[k] = hdeg[k - 1];
+      hubs.v[k] = hubs.v[k - 1];
+    }
+    hdeg[k] = deg;
+    hubs.v[k] = (uint32_t)v;
+  }
+  for (; nh < kReduceHubs; ++nh) hubs.v[nh] = hubs.v[0];
+
+  const size_t words = 2 * (size_t)((m + 63) / 64);
+  DevBuf table, bits;
+  cudaError_t e = table.reserve(sizeof(uint32_t) * (16 * (size_t)n + kReduceRounds + 1));
+  if (e == cudaSuccess) e = bits.reserve(sizeof(uint32_t) * words);
+  std::vector<uint32_t> keep;
+  if (e == cudaSuccess) {
+    keep.resize(words);
+    e = mark_useful_arcs(g->dg, hubs, table.as<uint32_t>(), table.as<unsigned>() + 16 * (size_t)n, bits.as<uint32_t>(),
+                         nullptr);
+    if (e == cudaSuccess) e = cudaMemcpy(keep.data(), bits.p, sizeof(uint32_t) * words, cudaMemcpyDeviceToHost);
+  }
+  table.release();
+  bits.release();
+  if (e == cudaErrorMemoryAllocation) {
+    (void)cudaGetLastError();
+    return cudaSuccess;
+  }
+  if (e != cudaSuccess) return e;
+
+  uint64_t kept = 0;
+  for (uint32_t w : keep) kept += (uint64_t)__builtin_popcount(w);
+  if (4 * kept > 3 * (uint64_t)m) return cudaSuccess;
+  std::vector<uint32_t> r_rp(rp.size()), r_adj((size_t)kept), r_wt((size_t)kept), hub_list;
+  uint64_t k = 0;
+  uint32_t max_deg = 0;
+  for (int64_t v = 0; v < n; ++v) {
+    const uint64_t k0 = k;
+    r_rp[(size_t)v] = (uint32_t)k;
+    for (uint64_t a = rp[(size_t)v], end = rp[(size_t)v + 1]; a < end;) {
+      // the word's bits from a on, cut at the row's end
+      uint32_t b = keep[a >> 5] >> (a & 31);
+      const uint64_t left = end - a, span = std::min<uint64_t>(32 - (a & 31), left);
+      if (span < 32) b &= (1u << span) - 1u;
+      for (; b; b &= b - 1) {
+        const uint64_t x = a + (uint64_t)__builtin_ctz(b);
+        r_adj[k] = adj[x];
+        r_wt[k] = wt[x];
+        ++k;
+      }
+      a += span;
+    }
+    const uint32_t deg = (uint32_t)(k - k0);
+    max_deg = std::max(max_deg, deg);
+    if (deg > kHubMin) hub_list.push_back((uint32_t)v);
+  }
+  r_rp[(size_t)n] = (uint32_t)k;
+
+  const size_t rp_elems = (size_t)g->nparts * (size_t)g->S + 64, arc_elems = (size_t)kept + 64;
+  e = g->s_rp.reserve(sizeof(uint32_t) * rp_elems);
+  if (e == cudaSuccess) e = g->s_adj.reserve(sizeof(uint32_t) * arc_elems);
+  if (e == cudaSuccess) e = g->s_wt.reserve(sizeof(uint32_t) * arc_elems);
+  if (e == cudaSuccess && !hub_list.empty()) e = g->s_hubs.reserve(sizeof(uint32_t) * hub_list.size());
+  if (e == cudaErrorMemoryAllocation) {
+    (void)cudaGetLastError();
+    release_reduced(g);
+    return cudaSuccess;
+  }
+  auto put = [&](DevBuf &d, const std::vector<uint32_t> &h, size_t elems) {
+    if (e == cudaSuccess && elems > h.size())
+      e = cudaMemset(d.as<uint32_t>() + h.size(), 0, sizeof(uint32_t) * (elems - h.size()));
+    if (e == cudaSuccess && !h.empty())
+      e = cudaMemcpy(d.p, h.data(), sizeof(uint32_t) * h.size(), cudaMemcpyHostToDevice);
+  };
+  put(g->s_rp, r_rp, rp_elems);
+  put(g->s_adj, r_adj, arc_elems);
+  put(g->s_wt, r_wt, arc_elems);
+  if (!hub_list.empty()) put(g->s_hubs, hub_list, hub_list.size());
+  if (e != cudaSuccess) return e;
+  g->s_dg = g->dg;
+  g->s_dg.m = kept;
+  g->s_dg.max_deg = max_deg;  // max_w stays the whole graph's: the overflow test covers every arc
+  g->s_dg.rp = g->s_rp.as<uint32_t>();
+  g->s_dg.adj = g->s_adj.as<uint32_t>();
+  g->s_dg.wt = g->s_wt.as<uint32_t>();
+  g->s_nhubs = (int32_t)hub_list.size();
+  g->reduced = true;
+  g->graph_bytes += sizeof(uint32_t) * ((size_t)n + 1 + 2 * (size_t)kept);
+  return cudaSuccess;
+}
+
 extern "C" fg_status fg_graph_create(int64_t n, int64_t m, const int64_t *row_ptr, const int32_t *col,
                                      const int32_t *w, uint32_t flags, fg_graph **out) {
   return fg_graph_create_ex(n, m, row_ptr, col, w, flags, nullptr, out);
@@ -254,6 +369,7 @@ extern "C" fg_status fg_graph_create_ex(int64_t n, int64_t m, const int64_t *row
   auto cleanup = [&](fg_status s) {
     g->rp.release(); g->adj.release(); g->wt.release(); g->orig.release(); g->intl.release();
     g->hubs.release();
+    release_reduced(g);
     delete g;
     return s;
   };
@@ -279,13 +395,18 @@ extern "C" fg_status fg_graph_create_ex(int64_t n, int64_t m, const int64_t *row
     CUDA_TRY_G(cudaMemset(g->wt.p, 0, sizeof(uint32_t) * arc_elems));
     if (m > 0) CUDA_TRY_G(cudaMemcpy(g->wt.p, i_wt.data(), sizeof(uint32_t) * (size_t)m, cudaMemcpyHostToDevice));
     g->graph_bytes += sizeof(uint32_t) * (size_t)m;
-    double sum = 0.0;
+    uint64_t sum = 0;  // locals: the loop keeps them in registers
+    uint32_t lo = 0xFFFFFFFFu, hi = 0;
     for (int64_t e = 0; e < m; ++e) {
-      sum += (double)i_wt[(size_t)e];
-      if (i_wt[(size_t)e] == 0u) g->has_zero_weight = true;
-      g->max_weight = std::max(g->max_weight, i_wt[(size_t)e]);
+      const uint32_t x = i_wt[(size_t)e];
+      sum += x;
+      lo = std::min(lo, x);
+      hi = std::max(hi, x);
     }
-    if (m > 0) g->mean_weight = sum / (double)m;
+    g->min_weight = m > 0 ? lo : 0u;
+    g->max_weight = hi;
+    g->has_zero_weight = m > 0 && lo == 0u;
+    if (m > 0) g->mean_weight = (double)sum / (double)m;
   }
   std::vector<uint32_t> hubs;
   for (int64_t v = 0; v < n; ++v) {
@@ -323,6 +444,13 @@ extern "C" fg_status fg_graph_create_ex(int64_t n, int64_t m, const int64_t *row
   d.wt = wt ? g->wt.as<uint32_t>() : nullptr;
   d.orig = identity ? nullptr : g->orig.as<int32_t>();
   d.intl = identity ? nullptr : g->intl.as<int32_t>();
+  if (wt) {
+    const cudaError_t e = build_reduced(g, i_rp, i_adj, i_wt);
+    if (e != cudaSuccess) {
+      cleanup(FG_OK);
+      return fail(FG_ERR_CUDA, "marking the arcs of shortest paths: %s", cudaGetErrorString(e));
+    }
+  }
   // the no-allocation entry point's scratch is placed on the device now, while
   // the caller's memory is still free (lazy module loading would otherwise
   // place it at that entry point's first call)
@@ -349,6 +477,7 @@ extern "C" fg_status fg_graph_destroy(fg_graph *g) {
     g->rp.release(); g->adj.release(); g->wt.release(); g->orig.release(); g->intl.release();
     g->deg.release();
     g->hubs.release();
+    release_reduced(g);
     g->bc.release_all();
     g->dfs.release_all();
     if (g->last_done) cudaEventDestroy(g->last_done);
@@ -621,7 +750,7 @@ fg_status run_batch_on(fg_graph *g, Workspace &ws, bool shared_ws, int grid_div,
     for (int64_t q0 = 0; q0 < nq; q0 += nbq) {
       const int64_t cnt_q = std::min<int64_t>(nbq, nq - q0);
       GroupArgs a;
-      a.g = g->dg;
+      set_group_graph(g, qtype, a);
       a.qtype = qtype;
       a.nq = (int32_t)cnt_q;
       a.G = Gq;
@@ -636,8 +765,6 @@ fg_status run_batch_on(fg_graph *g, Workspace &ws, bool shared_ws, int grid_div,
       a.hub_cap = (uint32_t)((uint64_t)a.ngroups * g->hub_chunks);
       a.hub_hi = Gq == 64 ? reinterpret_cast<uint32_t *>(a.items + a.hub_cap + (size_t)a.ngroups * (size_t)g->nparts)
                           : nullptr;
-      a.hubs = g->nhubs ? g->hubs.as<uint32_t>() : nullptr;
-      a.nhubs = g->nhubs;
       a.hub_chunk = kHubChunk;
       a.window = qtype == Q_SSSP && o.sched == FG_SCHED_PRIORITY ? o.sched_window : 0u;
       a.gbest = a.window ? ws.g_best.as<uint32_t>() : nullptr;
@@ -906,6 +1033,15 @@ int auto_group_size(const fg_graph *g, int qtype, int64_t nq, bool windowed) {
   while (G > 8 && (int64_t)(G / 2) >= nq) G /= 2;  // a small batch: the smallest group that holds it
   while (G > 8 && !group_fits(g->S, G)) G /= 2;
   return group_fits(g->S, G) ? G : 1;
+}
+
+void set_group_graph(const fg_graph *g, int qtype, GroupArgs &a) {
+  const bool red = qtype == Q_SSSP && g->reduced;
+  a.g = red ? g->s_dg : g->dg;
+  a.nhubs = red ? g->s_nhubs : g->nhubs;
+  a.hubs = a.nhubs ? (red ? g->s_hubs : g->hubs).as<uint32_t>() : nullptr;
+  a.all_rp = red ? g->dg.rp : nullptr;
+  a.all_wt = red ? g->dg.wt : nullptr;
 }
 
 fg_status report_error(fg_status s, const char *msg) {

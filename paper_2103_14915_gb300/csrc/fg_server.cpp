@@ -241,7 +241,7 @@ fg_status launch_slot_lane(fg_server *s, SlotLane &C) {
   }
   CUDA_TRY(cudaMemsetAsync(C.ctrl.p, 0, sizeof(Ctrl), C.stream));
   GroupArgs a;
-  a.g = g->dg;
+  set_group_graph(g, C.qtype, a);
   a.qtype = C.qtype;
   a.nq = C.nslots;
   a.G = C.G;
@@ -254,8 +254,6 @@ fg_status launch_slot_lane(fg_server *s, SlotLane &C) {
   a.dirty = C.dirty.as<uint32_t>();
   a.items = C.items.as<uint4>();
   a.hub_cap = (uint32_t)((uint64_t)C.ngroups * g->hub_chunks);
-  a.hubs = g->nhubs ? g->hubs.as<uint32_t>() : nullptr;
-  a.nhubs = g->nhubs;
   a.hub_chunk = kHubChunk;
   a.window = 0u;  // lanes of one group are of different ages: no shared window
   a.gbest = nullptr;
