@@ -125,3 +125,26 @@ def test_overflow_on_an_arc_that_was_left_out():
                 assert np.array_equal(got[0, :g0.n].astype(np.int64), want), (room, G)
         finally:
             fg.fg_graph_destroy(h)
+
+
+@pytest.mark.parametrize("weights,directed", [((1, 8), False), ((1, 255), True)])
+def test_dependencies_are_the_same(weights, directed):
+    """BC runs on the graph that SSSP runs on: the same tight arcs in the same
+    order. Small weights tie many paths."""
+    g = inputs.rmat(13, 16, seed=11, directed=directed, weights=weights)
+    srcs = np.concatenate([inputs.sources_uniform(g, 6, 5), [int(np.argmax(g.out_degree()))]]).astype(np.int32)
+    h, reduced = build(g, fg.FG_PART_RANGE)
+    try:
+        assert reduced
+        s_d = torch.from_numpy(srcs).to(DEV)
+        dist = torch.empty((len(srcs), g.n), dtype=torch.int32, device=DEV)
+        fg.check(fg.fg_sssp_batch(h, s_d, len(srcs), dist))
+        fg.check(fg.fg_sync())
+        bc = torch.empty(g.n, dtype=torch.float64, device=DEV)
+        st, info = fg.fg_bc_accumulate(h, s_d, len(srcs), dist, True, bc)
+        fg.check(st)
+        ref, sigma_max, exact = oracle.bc(g, srcs, True)
+        assert exact and info.inexact == 0 and info.sigma_max == sigma_max
+        assert np.array_equal(bc.cpu().numpy(), ref)
+    finally:
+        fg.fg_graph_destroy(h)
