@@ -907,7 +907,7 @@ __global__ void __launch_bounds__(kThreads, 3) engine_kernel(EngineArgs a) {
   }
   Ctrl *c = a.ctrl;
   // every block reads the generation before its first arrival, so all agree
-  unsigned gen = *reinterpret_cast<volatile unsigned *>(&c->bar_gen);
+  unsigned gen = barrier_generation(c);
   Counters ctr;
   // phase clock of block 0 (device time between device-wide barriers)
   uint64_t t_prev = (blockIdx.x == 0 && threadIdx.x == 0) ? global_ns() : 0ull;

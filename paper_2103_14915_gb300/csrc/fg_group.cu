@@ -293,7 +293,7 @@ __global__ void __launch_bounds__(kGThreads, 3) group_kernel(GroupArgs a) {
   constexpr int kB = group_batch(GQ);  // listed vertices per consumer batch
   uint32_t *sdv = g_smem + 2 * iw + (size_t)kGCons * 128u + (size_t)(producer ? 0 : wid) * (size_t)kB * (uint32_t)Gq;
   Ctrl *c = a.ctrl;
-  unsigned gen = *reinterpret_cast<volatile unsigned *>(&c->bar_gen);
+  unsigned gen = barrier_generation(c);
   uint32_t it_base = 0;   // items this block has gone through (both buffers), the same in every warp
   uint32_t tma_bits = 0;  // producer: phase parity of s_tma[0] (bit 0) and s_tma[1] (bit 1)
   uint32_t r32 = 0, i32 = 0, a32 = 0;  // per-item counters, folded into s_stat after each item

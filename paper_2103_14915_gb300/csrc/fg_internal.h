@@ -1,6 +1,7 @@
 // Internal structures shared by the host runtime and the CUDA kernels.
 #pragma once
 
+#include <cstddef>
 #include <cstdint>
 
 #include <cuda_runtime.h>
@@ -37,8 +38,6 @@ struct DevGraph {
 
 // Device control block of one batch launch (zeroed before each launch).
 struct Ctrl {
-  unsigned int bar_count;
-  unsigned int bar_gen;
   int status;                 // fg_status raised on the device (0 = ok)
   int abort;                  // set with status: every block leaves at its next check
   unsigned int item_next;     // work-claiming counter of the current round
@@ -52,7 +51,11 @@ struct Ctrl {
   unsigned long long arcs_read;  // graph arcs read (per query visit, or per group visit)
   unsigned int max_ops[2];       // largest buffer of the round, per round parity (max-operations scheduling)
   unsigned int g_exit;           // group engine, serve mode: the launch ends after this round
+  // arrivals at the device-wide barrier; top bit: leave (grid_barrier). In the
+  // second 128-byte line, which nothing that blocks compete for shares
+  unsigned long long bar;
 };
+static_assert(offsetof(Ctrl, bar) >= 128 && sizeof(Ctrl) <= 256, "control block");
 
 // Serve mode of the group engine (continuous batching): a mailbox in mapped
 // host memory. The host writes a slot's source, then a new sequence number;

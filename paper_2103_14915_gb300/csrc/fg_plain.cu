@@ -23,7 +23,7 @@ template <int QT>
 __global__ void __launch_bounds__(kPlainThreads) plain_kernel(PlainArgs a) {
   const DevGraph &g = a.g;
   Ctrl *c = a.ctrl;
-  unsigned gen = *reinterpret_cast<volatile unsigned *>(&c->bar_gen);
+  unsigned gen = barrier_generation(c);
   const uint32_t n = (uint32_t)g.n;
   const uint32_t tid = blockIdx.x * blockDim.x + threadIdx.x, nthr = gridDim.x * blockDim.x;
   const int lane = lane_id();
