@@ -106,9 +106,9 @@ typedef struct {
                                so one batch's copy to the host overlaps the next batch's
                                kernels when they run on different streams */
     int32_t query_batch;    /* queries per device launch; 0 = all (bounded by workspace) */
-    int32_t threads_per_vertex; /* SSSP/BFS expansion: 1 = one lane per frontier vertex (graphs
-                               with out-degree <= 8 only), 32 or 0 (default) = a warp shares
-                               a batch of 32 frontier vertices' arcs evenly */
+    int32_t threads_per_vertex; /* 0 (default), 1 or 32; the engine picks the form of SSSP/BFS
+                               expansion by the graph's out-degrees (arc records of fixed size up
+                               to 8, else a warp shares the arcs of 32 frontier vertices evenly) */
     int32_t group;          /* SSSP/BFS queries that share one partition visit lane by lane
                                (the query group): 8, 16, 32 or 64 = the group engine, whose state
                                keeps a group's values of one vertex in one line, so one access
@@ -257,9 +257,8 @@ enum { FG_QUERY_SSSP = 0, FG_QUERY_BFS = 1, FG_QUERY_PPR = 2 };
  * fg_opts.group); then, with one query per warp, FG_SCHED_PRIORITY windows from
  * wide to narrow -- multiples of the graph's mean arc weight for SSSP, levels
  * for BFS -- until one takes more than twice the best time, delta (yield
- * heuristic 2) of half and a quarter of the best window, and on graphs with
- * out-degree <= 8 lane-per-vertex expansion; with the group engine, SSSP
- * windows of 16 and 4 mean weights; last, for every kind with nq >= 64, half
+ * heuristic 2) of half and a quarter of the best window; with the group
+ * engine, SSSP windows of 16 and 4 mean weights; last, for every kind with nq >= 64, half
  * the batch per launch (query_batch). PPR keeps FIFO scheduling. best->group
  * is never 0: the automatic choice is resolved. The partition size is a graph
  * property: compare graphs created with different partition_vertices. src: DEVICE int32[nq] (the sample; a few hundred sources is

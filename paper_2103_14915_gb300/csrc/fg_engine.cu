@@ -37,7 +37,9 @@ constexpr uint32_t kMaxVisitSteps = 1u << 22;  // relax/push steps of one visit 
 constexpr uint32_t kBlockChunk = 16;            // work items a block claims at once
 constexpr uint32_t kTailChunk = 2;              // ... once fewer than 4 full chunks per block are left
 constexpr uint32_t kArenaChunk = 64;            // arena slots a warp reserves at once (>= 32)
-constexpr int kLaneMaxDeg = 8;                  // lane-per-vertex expansion for max out-degree <= 8
+constexpr int kUnroll = 4;                      // steps of 32 arcs with their loads in flight together
+constexpr uint32_t kMoreArcs = 0x8000u;         // of a queue entry
+constexpr int kExt = 64;                        // candidates for other partitions a warp gathers before it sends them
 
 // Per-warp counters. visits and edges are lane-uniform; spills and yields are
 // summed over the lanes when flushed.
@@ -45,21 +47,35 @@ struct Counters {
   unsigned long long visits = 0, edges = 0, spills = 0, yields = 0;
 };
 
-// Per-warp shared memory: the state slice and five bitmaps of S bits.
+// Per-warp shared memory of a PPR visit: the residuals and four bitmaps of S bits.
 struct WarpSmem {
-  uint32_t *d;      // [S] distances (u32) or residuals (f32 bits)
+  uint32_t *d;      // [S] residuals (f32 bits)
   uint32_t *cur;    // [nw] frontier being expanded
   uint32_t *nxt;    // [nw] frontier of the next step
-  uint32_t *far;    // [nw] values beyond the current in-visit window
   uint32_t *carry;  // [nw] left for a later visit (yield / spill)
   uint32_t *pfx;    // [nw] exclusive popcount prefix of cur
 };
 
+// Per-warp shared memory of an SSSP / BFS visit: the distances, a queue of the
+// vertices to expand, and four bitmaps of S bits.
+struct DistSmem {
+  uint32_t *d;      // [S] distances
+  uint16_t *ring;   // [S] queue of vertices to expand, each at most once; kMoreArcs: may have more than four arcs
+  uint32_t *inq;    // [nw] vertices in the queue
+  uint32_t *far;    // [nw] values at or beyond the in-visit window T when marked
+  uint32_t *carry;  // [nw] values at or beyond the visit's bound Ty when marked
+  uint32_t *spill;  // [nw] vertices whose candidates for other partitions did not fit
+  uint32_t *ext;    // [3 * kExt] candidates for other partitions: target, value, source
+};
+
 // Per-warp area in words, rounded up to 16 bytes so every warp's slice is
 // 16-byte aligned (the dynamic shared memory base is).
-__host__ __device__ inline size_t warp_smem_words(int S) {
-  return ((size_t)S + 5u * (size_t)(S / 32) + 3u) & ~(size_t)3u;
+__host__ __device__ inline size_t warp_smem_words(bool ppr, int S) {
+  const size_t nw = (size_t)(S / 32);
+  const size_t words = ppr ? (size_t)S + 4u * nw : (size_t)S + (size_t)S / 2u + 4u * nw + 3u * (size_t)kExt;
+  return (words + 3u) & ~(size_t)3u;
 }
+
 
 
 // ---------------------------------------------------------------------------
@@ -177,49 +193,6 @@ __device__ __forceinline__ uint32_t frontier_prefix(const WarpSmem &w, const Wor
 }
 
 // idx-th set bit of cur (0-based), using the prefix array.
-// Register form of the step's frontier, for partitions of at most 1024
-// vertices (at most one bitmap word per lane): lane l holds word l of cur,
-// the popcount prefix of the words before it, and the total. Selection then
-// needs shuffles only (no prefix words in shared memory, no warp sync).
-struct RegFrontier {
-  uint32_t word, ex, tot;
-};
-
-__device__ __forceinline__ RegFrontier reg_frontier(const WarpSmem &w, int nw, int lane) {
-  RegFrontier f;
-  f.word = lane < nw ? w.cur[lane] : 0u;
-  const uint32_t c = (uint32_t)__popc(f.word);
-  const uint32_t incl = warp_incl_scan(c);
-  f.ex = incl - c;
-  f.tot = __shfl_sync(kFull, incl, 31);
-  return f;
-}
-
-// Position of the r-th set bit (r counted from 0, r < popcount(x)), found by
-// halving: compare r with the popcount of the lower half at each width.
-__device__ __forceinline__ uint32_t nth_set_bit(uint32_t x, uint32_t r) {
-  uint32_t pos = 0;
-#pragma unroll
-  for (int wd = 16; wd; wd >>= 1) {
-    const uint32_t lo = (uint32_t)__popc(x & ((1u << wd) - 1u));
-    if (r >= lo) {
-      r -= lo;
-      x >>= wd;
-      pos += (uint32_t)wd;
-    }
-  }
-  return pos;
-}
-
-// Vertex (slice index) of frontier position idx < f.tot. Warp-collective:
-// every lane calls it (inactive lanes with idx = 0).
-__device__ __forceinline__ uint32_t reg_select(const RegFrontier &f, uint32_t idx) {
-  const int L = owner_lane(f.ex, idx);  // the lane whose word holds position idx
-  const uint32_t wL = __shfl_sync(kFull, f.word, L);
-  const uint32_t exL = __shfl_sync(kFull, f.ex, L);
-  return (uint32_t)L * 32u + nth_set_bit(wL, idx - exL);
-}
-
 __device__ __forceinline__ uint32_t frontier_select(const WarpSmem &w, int nw, uint32_t idx) {
   int lo = 0, hi = nw - 1;
   while (lo < hi) {
@@ -261,41 +234,167 @@ __device__ __forceinline__ bool arcs_in_range(const DevGraph &g, uint32_t e0, ui
   return (uint64_t)e0 + deg <= g.m;
 }
 
-__device__ __forceinline__ uint32_t relax_value(const EngineArgs &a, uint32_t d, uint32_t w) {
-  const uint64_t s64 = (uint64_t)d + (uint64_t)w;
-  if (s64 >= (uint64_t)kInf) {
+// The visit's queue: positions head .. tail - 1 of the ring (modulo S).
+struct Queue {
+  uint32_t head = 0, tail = 0;  // the same in every lane
+};
+
+// Shared-memory atomics with a result under a predicate (no branch): the old
+// value, or `none` where on is false.
+__device__ __forceinline__ uint32_t shared_min_if(bool on, uint32_t addr, uint32_t x, uint32_t none) {
+  uint32_t old = none;
+  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %3, 0;\n\t@q atom.shared.min.u32 %0, [%1], %2;\n\t}"
+               : "+r"(old) : "r"(addr), "r"(x), "r"((uint32_t)on) : "memory");
+  return old;
+}
+__device__ __forceinline__ uint32_t shared_or_if(bool on, uint32_t addr, uint32_t x, uint32_t none) {
+  uint32_t old = none;
+  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %3, 0;\n\t@q atom.shared.or.b32 %0, [%1], %2;\n\t}"
+               : "+r"(old) : "r"(addr), "r"(x), "r"((uint32_t)on) : "memory");
+  return old;
+}
+
+// K arcs a lane: from values dv to targets u (kInf: none; bit 31 = the target
+// has more than four arcs) over weights wt. A target in this partition is
+// lowered, marked in its set -- queue (nd < T), far window ([T, Ty)) or later
+// visit -- and, if it was not in it yet, put into the queue. A far or carry bit
+// stays when its vertex is lowered into the queue: the sets are held against
+// the values when they are read. out[k] = the target lies in another
+// partition. Every lane calls it.
+//
+// A step of a visit is one chain of dependent operations, and a branch of its
+// own for each arc would put the arcs' chains one after another; so the arcs go
+// side by side, predicated, with one vote each at the end.
+template <int QT, int K>
+__device__ __forceinline__ void relax_arcs(const EngineArgs &a, const DistSmem &w, Queue &qu, const uint32_t (&u)[K],
+                                           const uint32_t (&wt)[K], const uint32_t (&dv)[K], uint32_t p, uint32_t T,
+                                           uint32_t Ty, uint32_t (&nd)[K], bool (&out)[K]) {
+  const uint32_t S1 = (uint32_t)(a.g.S - 1), lt = (1u << lane_id()) - 1u;
+  const uint32_t s_d = smem_addr(w.d), s_inq = smem_addr(w.inq), s_far = smem_addr(w.far), s_carry = smem_addr(w.carry);
+  uint32_t old[K], was[K];
+  bool over = false;
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    nd[k] = dv[k] + (QT == Q_BFS ? 1u : wt[k]);
+    over |= u[k] != kInf && (nd[k] < dv[k] || nd[k] == kInf);
+  }
+  if (over) {  // 2^32 - 1 reached: saturate and report
     atomicCAS(&a.ctrl->status, 0, (int)FG_ERR_OVERFLOW);
-    return kInf - 1u;
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+      if (nd[k] < dv[k] || nd[k] == kInf) nd[k] = kInf - 1u;
   }
-  return (uint32_t)s64;
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const bool in = ((u[k] & 0x7FFFFFFFu) >> a.g.slog2) == p;
+    out[k] = u[k] != kInf && !in;
+    old[k] = shared_min_if(u[k] != kInf && in, s_d + (u[k] & S1) * 4u, nd[k], 0u);
+  }
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const uint32_t lu = u[k] & S1, set = nd[k] < T ? s_inq : (nd[k] < Ty ? s_far : s_carry);
+    was[k] = shared_or_if(nd[k] < old[k], set + (lu >> 5) * 4u, 1u << (lu & 31), kFull);
+  }
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const uint32_t lu = u[k] & S1;
+    const bool push = ((was[k] >> (lu & 31)) & 1u) == 0u && nd[k] < T;
+    const unsigned m = __ballot_sync(kFull, push);
+    if (push) w.ring[(qu.tail + (uint32_t)__popc(m & lt)) & S1] = (uint16_t)(lu | ((u[k] >> 31) << 15));
+    qu.tail += (uint32_t)__popc(m);
+  }
 }
 
-// Lower a partition-local vertex and route it: next step (< T), far window
-// ([T, Ty)) or a later visit (>= Ty), clearing the bit of its previous class.
-__device__ __forceinline__ void relax_local(const WarpSmem &w, uint32_t lu, uint32_t nd, uint32_t T, uint32_t Ty) {
-  const uint32_t bit = 1u << (lu & 31);
-  const uint32_t old = atomicMin(&w.d[lu], nd);
-  if (nd < old) {
-    if (nd < T) {
-      atomicOr(&w.nxt[lu >> 5], bit);
-      if (old != kInf && old >= T) {
-        if (old < Ty) atomicAnd(&w.far[lu >> 5], ~bit);
-        else atomicAnd(&w.carry[lu >> 5], ~bit);
-      }
-    } else if (nd < Ty) {
-      atomicOr(&w.far[lu >> 5], bit);
-      if (old != kInf && old >= Ty) atomicAnd(&w.carry[lu >> 5], ~bit);
-    } else {
-      atomicOr(&w.carry[lu >> 5], bit);
-    }
-  }
+// Put the set bits of a lane's word of inq into the queue. Every lane calls it.
+__device__ __forceinline__ void queue_bits(const DistSmem &w, Queue &qu, uint32_t bits, uint32_t first, uint32_t S1) {
+  const uint32_t c = (uint32_t)__popc(bits), incl = warp_incl_scan(c);
+  uint32_t at = qu.tail + incl - c;
+  for (; bits; bits &= bits - 1u) w.ring[at++ & S1] = (uint16_t)((first + (uint32_t)__ffs(bits) - 1u) | kMoreArcs);
+  qu.tail += __shfl_sync(kFull, incl, 31);
 }
 
 // ---------------------------------------------------------------------------
-// SSSP / BFS visit of one (partition, query) buffer.
+// Candidates for other partitions. An arc that leaves the partition needs the
+// target's committed value, a read from L2 or HBM, and on a road-like graph
+// one arc in twenty leaves: read on the spot, it would add its latency to
+// most steps of the visit's chain. So a visit puts such candidates (target,
+// value, source vertex) into the warp's list in shared memory and sends them
+// 32 at a time: drop those that do not lower the target, append the others to
+// the arena, and mark the source of one that does not fit for a later visit.
 // ---------------------------------------------------------------------------
-template <int QT, bool LANES>
-__device__ void visit_dist(const EngineArgs &a, const WarpSmem &w0, uint4 item, uint32_t qbound, const uint32_t *prp,
+struct ExtList {
+  uint32_t n = 0;  // held, the same in every lane, < 32 between calls
+};
+
+__device__ __forceinline__ void ext_send(const EngineArgs &a, const DistSmem &w, ExtList &x, uint32_t cnt, uint32_t q,
+                                         Counters &ctr, ArenaSlots &sl) {
+  const int lane = lane_id();
+  __syncwarp();
+  const bool mine = (uint32_t)lane < cnt;
+  const uint32_t u = mine ? w.ext[lane] : 0u, nd = mine ? w.ext[kExt + lane] : kInf,
+                 v = mine ? w.ext[2 * kExt + lane] : 0u;
+  const bool has = mine && nd < a.dist[(size_t)q * (size_t)a.g.n + u];
+  if (!emit_ops(a, has, (u >> a.g.slog2) * (uint32_t)a.nq + q, u & (uint32_t)(a.g.S - 1), nd, true, &sl)) {
+    atomicOr(&w.spill[v >> 5], 1u << (v & 31));
+    ctr.spills++;
+  }
+  const uint32_t left = x.n - cnt;  // < 32
+  uint32_t m0 = 0u, m1 = 0u, m2 = 0u;
+  if ((uint32_t)lane < left) {
+    m0 = w.ext[cnt + lane];
+    m1 = w.ext[kExt + cnt + lane];
+    m2 = w.ext[2 * kExt + cnt + lane];
+  }
+  __syncwarp();
+  if ((uint32_t)lane < left) {
+    w.ext[lane] = m0;
+    w.ext[kExt + lane] = m1;
+    w.ext[2 * kExt + lane] = m2;
+  }
+  x.n = left;
+  __syncwarp();
+}
+
+// Every lane calls it; lanes with `on` have a candidate.
+__device__ __forceinline__ void ext_add(const EngineArgs &a, const DistSmem &w, ExtList &x, bool on, uint32_t u,
+                                        uint32_t nd, uint32_t v, uint32_t q, Counters &ctr, ArenaSlots &sl) {
+  const unsigned m = __ballot_sync(kFull, on);
+  if (m == 0u) return;
+  if (on) {
+    const uint32_t at = x.n + (uint32_t)__popc(m & ((1u << lane_id()) - 1u));
+    w.ext[at] = u;
+    w.ext[kExt + at] = nd;
+    w.ext[2 * kExt + at] = v;
+  }
+  x.n += (uint32_t)__popc(m);
+  if (x.n >= 32u) ext_send(a, w, x, 32u, q, ctr, sl);
+}
+
+// ---------------------------------------------------------------------------
+// SSSP / BFS visit of one (partition, query) buffer. On a road-like graph a
+// visit expands few vertices at a time (some eleven of four arcs on the
+// 1024^2 grid) one after another, so its time is the length of the dependent
+// chain of a step, not its arcs. Vertices to expand wait in a first-in
+// first-out queue; a step takes up to 32 from its head, in one of two forms:
+//   PAIRS  graphs whose out-degrees are at most kPairSlots: the arcs of a
+//          vertex stand in a record of fixed size (g.pairs), read without
+//          offsets, scan or search. Two lanes take a vertex, two arcs each
+//          with one 16-byte load; the few vertices of more than four arcs
+//          take a second load. 16 vertices a step. (The three figures below
+//          in the other form: 67.0, 20.9 and 0.61 ms.)
+//   else   the arcs of 32 vertices are spread evenly over the lanes, kUnroll
+//          runs of 32 with their loads in flight together.
+// What a step spends is mostly warp-wide operations (35-65 cycles each for a
+// vote, a shuffle, a warp barrier, as for a shared-memory read) and branches, so
+// the queue is a list in shared memory rather than bitmaps searched with scans,
+// arcs go side by side (relax_arcs), and whatever is rare stands behind one
+// branch. On the 1024^2 grid (GB300; with bitmaps, two reads behind the offsets
+// and 32 arcs after another before): SSSP, 256 sources 82.0 -> 58.1 ms; BFS on
+// 701 x 1113, 100 sources 29.8 -> 17.9; one source on 41 x 48 0.92 -> 0.45. A
+// round ends with its longest visit: warps wait 60 % of their time there.
+// ---------------------------------------------------------------------------
+template <int QT, bool PAIRS>
+__device__ void visit_dist(const EngineArgs &a, const DistSmem &w, uint4 item, uint32_t qbound, const uint32_t *prp,
                            Counters &ctr, ArenaSlots &sl) {
   const DevGraph &g = a.g;
   const int lane = lane_id();
@@ -303,46 +402,40 @@ __device__ void visit_dist(const EngineArgs &a, const WarpSmem &w0, uint4 item, 
   const uint32_t nq = (uint32_t)a.nq;
   const uint32_t p = key / nq, q = key - p * nq;
   const int S = g.S, nw = S >> 5;
+  const uint32_t S1 = (uint32_t)(S - 1);
   const uint32_t base = p << g.slog2;
   const int Sp = min(S, g.n - (int)base);
   uint32_t *drow = a.dist + (size_t)q * (size_t)g.n;
-  WarpSmem w = w0;
-  const WordRange wr(nw, lane);
+  Queue qu;
+  ExtList xl;
 
   // 1. stage the query's slice of this partition (bypassing L1)
   load_slice(w.d, drow + base, Sp, lane);
   for (int i = Sp + lane; i < S; i += 32) w.d[i] = kInf;
-  for (int wd = lane; wd < nw; wd += 32) {
-    w.cur[wd] = 0u; w.nxt[wd] = 0u; w.far[wd] = 0u; w.carry[wd] = 0u;
-  }
-  // 2. vertices deferred by an earlier visit
   uint32_t *pend = a.pend + (size_t)key * (size_t)nw;
-  if (flags & 1u) {
-    for (int wd = lane; wd < nw; wd += 32) {
-      w.cur[wd] = __ldcg(pend + wd);
+  for (int wd = lane; wd < nw; wd += 32) {
+    // 2. vertices deferred by an earlier visit
+    uint32_t b = 0u;
+    if (flags & 1u) {
+      b = __ldcg(pend + wd);
       pend[wd] = 0u;
     }
+    w.inq[wd] = b; w.far[wd] = 0u; w.carry[wd] = 0u; w.spill[wd] = 0u;
   }
   __syncwarp();
   // 3. apply buffered operations; an operation is live iff it improves the value
   const uint2 *ops = a.b_op + off;
   for (uint32_t j = lane; j < cnt; j += 32) {
     const uint2 o = __ldcg(ops + j);
-    const uint32_t old = atomicMin(&w.d[o.x], o.y);
-    if (o.y < old) atomicOr(&w.cur[o.x >> 5], 1u << (o.x & 31));
+    if (o.y < atomicMin(&w.d[o.x], o.y)) atomicOr(&w.inq[o.x >> 5], 1u << (o.x & 31));
   }
+  __syncwarp();
+  for (int wd = lane; wd - lane < nw; wd += 32) queue_bits(w, qu, wd < nw ? w.inq[wd] : 0u, (uint32_t)wd * 32u, S1);
   __syncwarp();
   // 4. in-visit windows: values >= Ty wait for a later visit (yield heuristic 2);
   //    values in [T, Ty) wait for the window to advance (near/far order).
   uint32_t fmin = kInf;
-  for (int wd = wr.w0; wd < wr.w1; ++wd) {
-    uint32_t b = w.cur[wd];
-    while (b) {
-      const int t = __ffs(b) - 1;
-      b &= b - 1;
-      fmin = min(fmin, w.d[wd * 32 + t]);
-    }
-  }
+  for (uint32_t i = lane; i < qu.tail; i += 32) fmin = min(fmin, w.d[w.ring[i] & ~kMoreArcs]);
   fmin = warp_min_u32(fmin);
   if (fmin == kInf) return;  // every operation was stale: the slice is unchanged
   ctr.visits++;
@@ -352,206 +445,191 @@ __device__ void visit_dist(const EngineArgs &a, const WarpSmem &w0, uint4 item, 
   const uint32_t Ty = min(a.delta ? sat_add_u32(fmin, a.delta) : kInf, qbound);
   uint32_t T = a.bucket ? min(sat_add_u32(fmin, a.bucket), Ty) : Ty;
   if (T != kInf) {
-    for (int wd = wr.w0; wd < wr.w1; ++wd) {
-      uint32_t b = w.cur[wd], keep = 0u, fa = 0u, ca = 0u;
-      while (b) {
-        const int t = __ffs(b) - 1;
-        const uint32_t bit = 1u << t;
-        b &= b - 1;
-        const uint32_t d = w.d[wd * 32 + t];
-        if (d < T) keep |= bit; else if (d < Ty) fa |= bit; else ca |= bit;
+    const uint32_t n0 = qu.tail;  // at most S entries, from position 0: kept ones move to the front
+    qu.tail = 0;
+    for (uint32_t b0 = 0; b0 < n0; b0 += 32) {
+      const uint32_t i = b0 + (uint32_t)lane;
+      const uint32_t v = i < n0 ? w.ring[i] & ~kMoreArcs : 0u;
+      const uint32_t d = i < n0 ? w.d[v] : kInf;
+      __syncwarp();
+      const bool keep = i < n0 && d < T;
+      if (i < n0 && !keep) {
+        const uint32_t bit = 1u << (v & 31);
+        atomicAnd(&w.inq[v >> 5], ~bit);
+        atomicOr(&(d < Ty ? w.far : w.carry)[v >> 5], bit);
       }
-      w.cur[wd] = keep; w.far[wd] |= fa; w.carry[wd] |= ca;
+      const unsigned m = __ballot_sync(kFull, keep);
+      if (keep) w.ring[qu.tail + (uint32_t)__popc(m & ((1u << lane) - 1u))] = (uint16_t)(v | kMoreArcs);
+      qu.tail += (uint32_t)__popc(m);
     }
     __syncwarp();
   }
 
-  uint64_t vis_edges = 0;
-  bool stopped = false;
-  uint32_t steps = 0;
+  const bool a_yields = a.yield_edges != 0;
+  uint32_t steps = 0, arcs = 0;  // arcs: of this lane
   for (;;) {
-    // bounded loop: a visit can never spin forever
-    if (++steps > kMaxVisitSteps || ((steps & 255u) == 0 && ld_volatile_i32(&a.ctrl->abort))) {
-      if (steps > kMaxVisitSteps) raise_status(a.ctrl, FG_ERR_TIMEOUT, kSiteVisit);
-      stopped = true;
-      break;
-    }
-    uint32_t F;
-    RegFrontier rf;
-    const bool reg_front = nw <= 32;
-    if (LANES) {
-      uint32_t cntl = 0;
-      for (int wd = wr.w0; wd < wr.w1; ++wd) cntl += __popc(w.cur[wd]);
-      F = __reduce_add_sync(kFull, cntl);
-    } else if (reg_front) {
-      rf = reg_frontier(w, nw, lane);
-      F = rf.tot;
-    } else {
-      F = frontier_prefix(w, wr);
-    }
-    if (F == 0) {
-      // advance the in-visit window to the smallest far value
-      uint32_t fm = kInf;
-      for (int wd = wr.w0; wd < wr.w1; ++wd) {
-        uint32_t b = w.far[wd];
-        while (b) {
-          const int t = __ffs(b) - 1;
-          b &= b - 1;
-          fm = min(fm, w.d[wd * 32 + t]);
-        }
+    // everything but taking a step stands behind one branch
+    if ((qu.head == qu.tail) | (++steps % 256u == 0u) | a_yields | arena_pressed(a, sl.seen)) {
+      // bounded loop: a visit can never spin forever
+      if (steps > kMaxVisitSteps) {
+        raise_status(a.ctrl, FG_ERR_TIMEOUT, kSiteVisit);
+        break;
       }
-      fm = warp_min_u32(fm);
-      if (fm == kInf) break;
-      T = a.bucket ? min(sat_add_u32(fm, a.bucket), Ty) : Ty;
-      for (int wd = wr.w0; wd < wr.w1; ++wd) {
-        uint32_t b = w.far[wd], mv = 0u;
-        while (b) {
-          const int t = __ffs(b) - 1;
-          b &= b - 1;
-          if (w.d[wd * 32 + t] < T) mv |= 1u << t;
+      if (steps % 256u == 0u && ld_volatile_i32(&a.ctrl->abort)) break;
+      if (qu.head == qu.tail) {
+        // advance the in-visit window to the smallest far value; a vertex whose
+        // value fell below the window since it was marked has been queued then
+        uint32_t fm = kInf;
+        if (a.bucket) {
+          for (int wd = lane; wd < nw; wd += 32) {
+            uint32_t b = w.far[wd], drop = 0u;
+            while (b) {
+              const int t = __ffs(b) - 1;
+              b &= b - 1;
+              const uint32_t d = w.d[wd * 32 + t];
+              if (d < T) drop |= 1u << t;
+              else fm = min(fm, d);
+            }
+            w.far[wd] &= ~drop;
+          }
+          fm = warp_min_u32(fm);
         }
-        w.far[wd] &= ~mv;
-        w.cur[wd] |= mv;
-      }
-      __syncwarp();
-      continue;
-    }
-    if (a.yield_edges && vis_edges >= a.yield_edges) {  // yield heuristic 1
-      stopped = true;
-      break;
-    }
-    if (arena_pressed(a, sl.seen)) {  // leave the rest of the visit to the next round
-      stopped = true;
-      break;
-    }
-    if (LANES) {
-      // low-degree graphs: each lane expands the frontier vertices of its own
-      // bitmap words, loading all arcs of a vertex at once
-      const int per = (nw + 31) >> 5;
-      for (int k = 0; k < per; ++k) {
-        const int wd = wr.w0 + k;
-        uint32_t b = (wd < wr.w1) ? w.cur[wd] : 0u;
-        while (__any_sync(kFull, b != 0u)) {
-          uint32_t v = 0, dv = 0, e0 = 0, deg = 0;
-          if (b) {
-            const int t = __ffs(b) - 1;
-            b &= b - 1;
-            v = (uint32_t)wd * 32u + (uint32_t)t;
-            dv = w.d[v];
-            e0 = prp[v];
-            deg = prp[v + 1] - e0;
-            if (deg > (uint32_t)kLaneMaxDeg || !arcs_in_range(g, e0, deg)) {  // inconsistent view: skip
-              raise_status(a.ctrl, FG_ERR_CUDA, kSiteDegree);
-              deg = 0;
+        if (fm == kInf) break;
+        T = min(sat_add_u32(fm, a.bucket), Ty);
+        for (int wd = lane; wd - lane < nw; wd += 32) {
+          uint32_t mv = 0u;
+          if (wd < nw) {
+            for (uint32_t b = w.far[wd]; b; b &= b - 1) {
+              const int t = __ffs(b) - 1;
+              if (w.d[wd * 32 + t] < T) mv |= 1u << t;
             }
+            w.far[wd] &= ~mv;
+            w.inq[wd] |= mv;
           }
-          vis_edges += __reduce_add_sync(kFull, deg);
-          uint32_t u[kLaneMaxDeg], nd[kLaneMaxDeg];
-#pragma unroll
-          for (int j = 0; j < kLaneMaxDeg; ++j) {
-            u[j] = 0u;
-            nd[j] = 0u;
-            if ((uint32_t)j < deg) {
-              u[j] = g.adj[e0 + j];
-              const uint32_t wgt = (QT == Q_BFS || g.wt == nullptr) ? 1u : g.wt[e0 + j];
-              nd[j] = relax_value(a, dv, wgt);
-            }
-          }
-          uint32_t extm = 0u;
-#pragma unroll
-          for (int j = 0; j < kLaneMaxDeg; ++j) {
-            if ((uint32_t)j < deg) {
-              if ((u[j] >> g.slog2) == p) {
-                relax_local(w, u[j] & (uint32_t)(S - 1), nd[j], T, Ty);
-              } else if (nd[j] < a.dist[(size_t)q * (size_t)g.n + u[j]]) {
-                extm |= 1u << j;
-              }
-            }
-          }
-          if (__any_sync(kFull, extm != 0u)) {
-#pragma unroll
-            for (int j = 0; j < kLaneMaxDeg; ++j) {
-              const bool e = (extm >> j) & 1u;
-              const uint32_t pk = (u[j] >> g.slog2) * nq + q;
-              if (!emit_ops(a, e, pk, u[j] & (uint32_t)(S - 1), nd[j], true, &sl)) {
-                atomicOr(&w.carry[v >> 5], 1u << (v & 31));
-                ctr.spills++;
-              }
-            }
-          }
-        }
-      }
-      __syncwarp();
-    } else {
-      // any degree distribution: the batch's arcs are spread evenly over the lanes
-      for (uint32_t b0 = 0; b0 < F; b0 += 32) {
-        const uint32_t idx = b0 + (uint32_t)lane;
-        uint32_t v = 0, dv = 0, a0 = 0, deg = 0;
-        if (reg_front) v = reg_select(rf, idx < F ? idx : 0u);
-        if (idx < F) {
-          if (!reg_front) v = frontier_select(w, nw, idx);
-          dv = w.d[v];
-          a0 = prp[v];
-          deg = prp[v + 1] - a0;
-          if (deg > g.max_deg || !arcs_in_range(g, a0, deg)) {  // inconsistent view: skip
-            raise_status(a.ctrl, FG_ERR_CUDA, kSiteDegree);
-            deg = 0;
-          }
-        }
-        const uint32_t incl = warp_incl_scan(deg);
-        const uint32_t exd = incl - deg;
-        const uint32_t tot = __shfl_sync(kFull, incl, 31);
-        vis_edges += tot;
-        for (uint32_t j = 0; j < tot; j += 32) {
-          const uint32_t t = j + (uint32_t)lane;
-          const bool has = t < tot;
-          const int L = owner_lane(exd, has ? t : 0u);
-          const uint32_t eL = __shfl_sync(kFull, a0, L) + (t - __shfl_sync(kFull, exd, L));
-          const uint32_t du = __shfl_sync(kFull, dv, L);
-          const uint32_t vL = __shfl_sync(kFull, v, L);
-          uint32_t u = 0, nd = 0;
-          bool ext = false;
-          if (has) {
-            u = g.adj[eL];
-            const uint32_t wgt = (QT == Q_BFS || g.wt == nullptr) ? 1u : g.wt[eL];
-            nd = relax_value(a, du, wgt);
-            if ((u >> g.slog2) == p) {
-              relax_local(w, u & (uint32_t)(S - 1), nd, T, Ty);
-            } else {
-              ext = nd < a.dist[(size_t)q * (size_t)g.n + u];
-            }
-          }
-          const uint32_t pk = (u >> g.slog2) * nq + q;
-          if (!emit_ops(a, ext, pk, u & (uint32_t)(S - 1), nd, true, &sl)) {
-            atomicOr(&w.carry[vL >> 5], 1u << (vL & 31));
-            ctr.spills++;
-          }
+          queue_bits(w, qu, mv, (uint32_t)wd * 32u, S1);
         }
         __syncwarp();
+        continue;
+      }
+      // yield heuristic 1, or arena pressure: leave the rest to a later visit
+      if ((a_yields && __reduce_add_sync(kFull, arcs) >= a.yield_edges) || arena_pressed(a, sl.seen)) break;
+    }
+    const uint32_t F = min(qu.tail - qu.head, PAIRS ? 16u : 32u);
+    // A vertex leaves the queue before its value is read, so that a later fall
+    // queues it again.
+    if (PAIRS) {
+      const uint32_t i = (uint32_t)lane >> 1;
+      uint32_t v = 0, dv = 0;
+      uint4 r = make_uint4(kInf, 0u, kInf, 0u), r2 = r;
+      bool more = false;
+      if (i < F) {
+        const uint32_t en = w.ring[(qu.head + i) & S1];
+        v = en & ~kMoreArcs;
+        more = (en & kMoreArcs) != 0u;
+        const uint4 *rec = reinterpret_cast<const uint4 *>(g.pairs) + (size_t)(base + v) * (kPairSlots / 2) + (lane & 1);
+        r = __ldg(rec);
+        if (more) r2 = __ldg(rec + 2);
+        if (!(lane & 1)) atomicAnd(&w.inq[v >> 5], ~(1u << (v & 31)));
+      }
+      qu.head += F;
+      const bool four = __any_sync(kFull, more);
+      __syncwarp();  // both lanes of a vertex read its value after it has left the queue
+      if (i < F) dv = w.d[v];
+      const uint32_t u[2] = {r.x, r.z}, wt[2] = {r.y, r.w}, from[2] = {dv, dv};
+      uint32_t nd[2], nd2[2] = {kInf, kInf};
+      bool out[2], out2[2] = {false, false};
+      arcs += (r.x != kInf ? 1u : 0u) + (r.z != kInf ? 1u : 0u);
+      relax_arcs<QT, 2>(a, w, qu, u, wt, from, p, T, Ty, nd, out);
+      const uint32_t u2[2] = {r2.x, r2.z}, wt2[2] = {r2.y, r2.w};
+      if (four) {
+        arcs += (r2.x != kInf ? 1u : 0u) + (r2.z != kInf ? 1u : 0u);
+        relax_arcs<QT, 2>(a, w, qu, u2, wt2, from, p, T, Ty, nd2, out2);
+      }
+      if (__any_sync(kFull, out[0] || out[1] || out2[0] || out2[1])) {
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          ext_add(a, w, xl, out[k], u[k] & 0x7FFFFFFFu, nd[k], v, q, ctr, sl);
+          ext_add(a, w, xl, out2[k], u2[k] & 0x7FFFFFFFu, nd2[k], v, q, ctr, sl);
+        }
+      }
+    } else {
+      uint32_t v = 0, dv = 0, a0 = 0, deg = 0;
+      if ((uint32_t)lane < F) {
+        v = w.ring[(qu.head + (uint32_t)lane) & S1] & ~kMoreArcs;
+        a0 = prp[v];
+        deg = prp[v + 1] - a0;
+        if (deg > g.max_deg || !arcs_in_range(g, a0, deg)) {  // inconsistent view: skip
+          raise_status(a.ctrl, FG_ERR_CUDA, kSiteDegree);
+          deg = 0;
+        }
+        atomicAnd(&w.inq[v >> 5], ~(1u << (v & 31)));
+      }
+      qu.head += F;
+      __syncwarp();
+      if ((uint32_t)lane < F) dv = w.d[v];
+      const uint32_t incl = warp_incl_scan(deg);
+      const uint32_t exd = incl - deg;
+      const uint32_t tot = __shfl_sync(kFull, incl, 31);
+      arcs += deg;
+      for (uint32_t j = 0; j < tot; j += 32u * kUnroll) {
+        uint32_t u[kUnroll], wt[kUnroll], own[kUnroll];
+#pragma unroll
+        for (int k = 0; k < kUnroll; ++k) {
+          u[k] = kInf;
+          wt[k] = 1u;
+          own[k] = 0u;
+          if (j + 32u * (uint32_t)k < tot) {  // warp-uniform
+            const uint32_t t = j + 32u * (uint32_t)k + (uint32_t)lane;
+            const bool has = t < tot;
+            const int L = owner_lane(exd, has ? t : 0u);
+            const uint32_t eL = __shfl_sync(kFull, a0, L) + (t - __shfl_sync(kFull, exd, L));
+            own[k] = (uint32_t)L;
+            if (has) {
+              u[k] = g.adj[eL];
+              if (QT != Q_BFS && g.wt != nullptr) wt[k] = g.wt[eL];
+            }
+          }
+        }
+        uint32_t du[kUnroll], nd[kUnroll];
+        bool out[kUnroll];
+#pragma unroll
+        for (int k = 0; k < kUnroll; ++k) du[k] = __shfl_sync(kFull, dv, (int)own[k]);
+        relax_arcs<QT, kUnroll>(a, w, qu, u, wt, du, p, T, Ty, nd, out);
+        bool any_out = false;
+#pragma unroll
+        for (int k = 0; k < kUnroll; ++k) any_out |= out[k];
+        if (__any_sync(kFull, any_out)) {
+#pragma unroll
+          for (int k = 0; k < kUnroll; ++k)
+            ext_add(a, w, xl, out[k], u[k], nd[k], __shfl_sync(kFull, v, (int)own[k]), q, ctr, sl);
+        }
       }
     }
-    // retire the expanded frontier; the next step expands nxt
-    for (int wd = wr.w0; wd < wr.w1; ++wd) w.cur[wd] = 0u;
-    __syncwarp();
-    uint32_t *tmp = w.cur; w.cur = w.nxt; w.nxt = tmp;
+    __syncwarp();  // the queue's new entries are read by the next step
   }
-  ctr.edges += vis_edges;
+  ctr.edges += __reduce_add_sync(kFull, arcs);
+  if (xl.n > 0u) ext_send(a, w, xl, xl.n, q, ctr, sl);
+  __syncwarp();
 
-  // 5. leftovers -> pending bitmap of this buffer
+  // 5. leftovers -> pending bitmap of this buffer: what is still queued (the
+  // visit stopped early), values beyond the bounds, spilled vertices. A carry
+  // bit whose value has fallen below Ty since went through the queue, a far
+  // one below T as well.
   uint32_t cmin = kInf;
   bool any = false;
-  for (int wd = wr.w0; wd < wr.w1; ++wd) {
-    uint32_t b = w.carry[wd];
-    if (stopped) b |= w.cur[wd] | w.nxt[wd] | w.far[wd];
+  for (int wd = lane; wd < nw; wd += 32) {
+    uint32_t b = w.inq[wd] | w.spill[wd];
+    uint32_t late = (w.carry[wd] | w.far[wd]) & ~b;
+    for (uint32_t x = b | late; x; x &= x - 1) {
+      const int t = __ffs(x) - 1;
+      const uint32_t bit = 1u << t, d = w.d[wd * 32 + t];
+      if ((late & bit) && d < T) continue;
+      b |= bit;
+      cmin = min(cmin, d);
+    }
     if (b) {
       any = true;
       pend[wd] = b;
-      uint32_t bb = b;
-      while (bb) {
-        const int t = __ffs(bb) - 1;
-        bb &= bb - 1;
-        cmin = min(cmin, w.d[wd * 32 + t]);
-      }
     }
   }
   any = __any_sync(kFull, any);
@@ -883,7 +961,7 @@ __device__ uint32_t claim_item(Ctrl *c, unsigned long long *claim, volatile int 
   }
 }
 
-template <int QT>
+template <int QT, bool PAIRS>
 __global__ void __launch_bounds__(kThreads, 3) engine_kernel(EngineArgs a) {
   extern __shared__ __align__(16) uint32_t smem_dyn[];
   __shared__ unsigned long long s_scan[kWarps + 1];
@@ -895,15 +973,25 @@ __global__ void __launch_bounds__(kThreads, 3) engine_kernel(EngineArgs a) {
 
   const int lane = lane_id(), wid = threadIdx.x >> 5;
   const int S = a.g.S, nw = S >> 5;
-  WarpSmem w;
+  WarpSmem w;   // PPR
+  DistSmem wd;  // SSSP, BFS
   {
-    uint32_t *b = smem_dyn + (size_t)wid * warp_smem_words(S);
-    w.d = b;
-    w.cur = b + S;
-    w.nxt = w.cur + nw;
-    w.far = w.nxt + nw;
-    w.carry = w.far + nw;
-    w.pfx = w.carry + nw;
+    uint32_t *b = smem_dyn + (size_t)wid * warp_smem_words(kPPR, S);
+    if (kPPR) {
+      w.d = b;
+      w.cur = b + S;
+      w.nxt = w.cur + nw;
+      w.carry = w.nxt + nw;
+      w.pfx = w.carry + nw;
+    } else {
+      wd.d = b;
+      wd.ring = reinterpret_cast<uint16_t *>(b + S);
+      wd.inq = b + S + S / 2;
+      wd.far = wd.inq + nw;
+      wd.carry = wd.far + nw;
+      wd.spill = wd.carry + nw;
+      wd.ext = wd.spill + nw;
+    }
   }
   Ctrl *c = a.ctrl;
   // every block reads the generation before its first arrival, so all agree
@@ -1204,8 +1292,7 @@ __global__ void __launch_bounds__(kThreads, 3) engine_kernel(EngineArgs a) {
           const uint32_t q = it.x - p * (uint32_t)a.nq;
           const uint32_t qbound =
               a.sched == FG_SCHED_PRIORITY ? sat_add_u32(__ldcg(qb_cur + q), a.sched_window) : kInf;
-          if (a.lanes) visit_dist<QT, true>(a, w, it, qbound, prp, ctr, sl);
-          else visit_dist<QT, false>(a, w, it, qbound, prp, ctr, sl);
+          visit_dist<QT, PAIRS>(a, wd, it, qbound, prp, ctr, sl);
         }
       }
       release_slots(a, sl);  // before the barrier: SCATTER reads every reserved slot
@@ -1282,18 +1369,43 @@ __global__ void __launch_bounds__(256) permute_out_kernel(const uint32_t *state,
 // ---------------------------------------------------------------------------
 // Launchers
 // ---------------------------------------------------------------------------
-static const void *engine_fn(int qtype) {
+// The arc records of a graph whose out-degrees are at most kPairSlots: left
+// packed, the rest kInf; bit 31 of a target = it has more than four arcs itself
+// (its record's second half is then read with the first).
+__global__ void __launch_bounds__(256) pair_records_kernel(DevGraph g, uint2 *out) {
+  const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  const int64_t v = i / kPairSlots;
+  const uint32_t k = (uint32_t)(i % kPairSlots);
+  if (v >= (int64_t)g.nparts * g.S) return;
+  uint2 r = make_uint2(kInf, 0u);
+  if (v < g.n) {
+    const uint32_t e = g.rp[v], deg = g.rp[v + 1] - e;
+    if (k < deg) {
+      const uint32_t u = g.adj[e + k];
+      r = make_uint2(u | (g.rp[u + 1] - g.rp[u] > 4u ? 0x80000000u : 0u), g.wt ? g.wt[e + k] : 1u);
+    }
+  }
+  out[i] = r;
+}
+
+cudaError_t launch_pair_records(const DevGraph &g, uint2 *out, cudaStream_t s) {
+  const int64_t total = (int64_t)g.nparts * g.S * kPairSlots;
+  pair_records_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(g, out);
+  return cudaGetLastError();
+}
+
+static const void *engine_fn(int qtype, bool pairs) {
   switch (qtype) {
-    case Q_SSSP: return (const void *)engine_kernel<Q_SSSP>;
-    case Q_BFS: return (const void *)engine_kernel<Q_BFS>;
-    default: return (const void *)engine_kernel<Q_PPR>;
+    case Q_SSSP: return pairs ? (const void *)engine_kernel<Q_SSSP, true> : (const void *)engine_kernel<Q_SSSP, false>;
+    case Q_BFS: return pairs ? (const void *)engine_kernel<Q_BFS, true> : (const void *)engine_kernel<Q_BFS, false>;
+    default: return (const void *)engine_kernel<Q_PPR, false>;
   }
 }
 
-cudaError_t engine_grid_size(int qtype, int S, int *blocks, int *threads, size_t *smem) {
-  const void *fn = engine_fn(qtype);
+cudaError_t engine_grid_size(int qtype, bool pairs, int S, int *blocks, int *threads, size_t *smem) {
+  const void *fn = engine_fn(qtype, pairs);
   *threads = kThreads;
-  *smem = (size_t)kWarps * warp_smem_words(S) * sizeof(uint32_t);
+  *smem = (size_t)kWarps * warp_smem_words(qtype == Q_PPR, S) * sizeof(uint32_t);
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem);
   if (e != cudaSuccess) return e;
   int per_sm = 0, dev = 0, sms = 0;
@@ -1309,7 +1421,7 @@ cudaError_t engine_grid_size(int qtype, int S, int *blocks, int *threads, size_t
 cudaError_t launch_engine(const EngineArgs &a, int blocks, int threads, size_t smem, cudaStream_t s) {
   EngineArgs copy = a;
   void *args[] = {(void *)&copy};
-  return cudaLaunchCooperativeKernel(engine_fn(a.qtype), dim3(blocks), dim3(threads), args, smem, s);
+  return cudaLaunchCooperativeKernel(engine_fn(a.qtype, a.g.pairs != nullptr), dim3(blocks), dim3(threads), args, smem, s);
 }
 
 cudaError_t launch_ppr_finalize(const EngineArgs &a, double *mass, float *p_out, float *r_out, cudaStream_t s) {

@@ -126,6 +126,7 @@ struct fg_graph {
   bool weighted = false;
   int device = 0;
   fg::DevBuf rp, adj, wt, orig, intl;
+  fg::DevBuf pairs;                // arc records of the query-major engine (out-degrees up to kPairSlots)
   fg::DevBuf deg;                  // out-degree per original id (built by the first fg_ncp_sweep)
   fg::BcWorkspace bc;              // fg_bc_accumulate scratch (guarded by mu)
   fg::DfsWorkspace dfs;            // fg_dfs_batch scratch (guarded by mu)

@@ -32,9 +32,14 @@ struct DevGraph {
   const uint32_t *rp = nullptr;    // [n+1] arc offsets
   const uint32_t *adj = nullptr;   // [m] internal target ids
   const uint32_t *wt = nullptr;    // [m] weights, or null (unit)
+  const uint2 *pairs = nullptr;    // [nparts * S][kPairSlots] (target, weight) records, or null (fg_engine.cu)
   const int32_t *orig = nullptr;   // [n] internal -> original id, or null (identity)
   const int32_t *intl = nullptr;   // [n] original -> internal id, or null (identity)
 };
+
+// Arcs of a vertex's record, for graphs of out-degrees up to this: 64 bytes a
+// vertex, against 34 for the offsets and arcs of a grid of 3.8 arcs a vertex.
+constexpr int kPairSlots = 8;
 
 // Device control block of one batch launch (zeroed before each launch).
 struct Ctrl {
@@ -108,7 +113,6 @@ struct EngineArgs {
   uint64_t yield_edges = 0;
   uint32_t max_rounds = 0;
   uint64_t watchdog_ns = 0;
-  uint32_t lanes = 0;  // 1: lane-per-vertex expansion (max out-degree <= 8)
 };
 
 // Group engine (fg_group.cu): G queries per group, lanes = queries. State is
@@ -175,8 +179,9 @@ struct PlainArgs {
 };
 
 // kernel launchers (fg_engine.cu / fg_plain.cu); return the CUDA error of the launch
-cudaError_t engine_grid_size(int qtype, int S, int *blocks, int *threads, size_t *smem);
+cudaError_t engine_grid_size(int qtype, bool pairs, int S, int *blocks, int *threads, size_t *smem);
 cudaError_t launch_engine(const EngineArgs &a, int blocks, int threads, size_t smem, cudaStream_t s);
+cudaError_t launch_pair_records(const DevGraph &g, uint2 *out, cudaStream_t s);
 cudaError_t launch_ppr_finalize(const EngineArgs &a, double *mass, float *p_out, float *r_out, cudaStream_t s);
 cudaError_t launch_permute_out(const uint32_t *state, uint32_t *out, const int32_t *orig, int64_t n, int64_t rows,
                                cudaStream_t s);

@@ -369,6 +369,7 @@ extern "C" fg_status fg_graph_create_ex(int64_t n, int64_t m, const int64_t *row
   auto cleanup = [&](fg_status s) {
     g->rp.release(); g->adj.release(); g->wt.release(); g->orig.release(); g->intl.release();
     g->hubs.release();
+    g->pairs.release();
     release_reduced(g);
     delete g;
     return s;
@@ -444,6 +445,21 @@ extern "C" fg_status fg_graph_create_ex(int64_t n, int64_t m, const int64_t *row
   d.wt = wt ? g->wt.as<uint32_t>() : nullptr;
   d.orig = identity ? nullptr : g->orig.as<int32_t>();
   d.intl = identity ? nullptr : g->intl.as<int32_t>();
+  if (m > 0 && g->max_degree <= (uint32_t)kPairSlots) {
+    // road-like: arc records for the query-major engine (without memory for
+    // them it takes the arcs through their offsets)
+    cudaError_t e = g->pairs.reserve(sizeof(uint2) * (size_t)kPairSlots * (size_t)g->nparts * (size_t)S);
+    if (e == cudaSuccess) e = launch_pair_records(d, g->pairs.as<uint2>(), nullptr);
+    if (e == cudaSuccess) {
+      d.pairs = g->pairs.as<uint2>();
+      g->graph_bytes += sizeof(uint2) * (size_t)kPairSlots * (size_t)n;
+    } else if (e == cudaErrorMemoryAllocation) {
+      (void)cudaGetLastError();
+    } else {
+      cleanup(FG_OK);
+      return fail(FG_ERR_CUDA, "arc records: %s", cudaGetErrorString(e));
+    }
+  }
   if (wt) {
     const cudaError_t e = build_reduced(g, i_rp, i_adj, i_wt);
     if (e != cudaSuccess) {
@@ -477,6 +493,7 @@ extern "C" fg_status fg_graph_destroy(fg_graph *g) {
     g->rp.release(); g->adj.release(); g->wt.release(); g->orig.release(); g->intl.release();
     g->deg.release();
     g->hubs.release();
+    g->pairs.release();
     release_reduced(g);
     g->bc.release_all();
     g->dfs.release_all();
@@ -788,7 +805,7 @@ fg_status run_batch_on(fg_graph *g, Workspace &ws, bool shared_ws, int grid_div,
                                      : std::min<uint64_t>(1ull << 29, std::max<uint64_t>(1ull << 22, 128 * K));
     e_cap = std::min<uint64_t>(std::max<uint64_t>(e_cap, (uint64_t)nb), 1ull << 31);
     if (g->engine_qtype != qtype) {
-      CUDA_TRY(engine_grid_size(qtype, g->S, &g->engine_blocks, &g->engine_threads, &g->engine_smem));
+      CUDA_TRY(engine_grid_size(qtype, g->dg.pairs != nullptr, g->S, &g->engine_blocks, &g->engine_threads, &g->engine_smem));
       g->engine_qtype = qtype;
     }
     fg_status st = ensure_engine_ws(g, ws, qtype, nb, e_cap, need_r, g->engine_blocks);
@@ -840,9 +857,6 @@ fg_status run_batch_on(fg_graph *g, Workspace &ws, bool shared_ws, int grid_div,
       a.yield_edges = o.yield_edges;
       a.max_rounds = max_rounds;
       a.watchdog_ns = watchdog_ns;
-      // lane-per-vertex expansion only on request (measured slower than the
-      // warp-shared merge-path on the road-like grid)
-      a.lanes = (o.threads_per_vertex == 1 && g->max_degree <= 8) ? 1u : 0u;
       CUDA_TRY(launch_engine(a, blocks, g->engine_threads, g->engine_smem, stream));
       ++launches;
       if (qtype == Q_PPR) {

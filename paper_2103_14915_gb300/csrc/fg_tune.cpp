@@ -9,8 +9,7 @@
 //     candidates are scaled by the graph's mean arc weight (SSSP) or counted in
 //     levels (BFS) and tried from the widest down until one takes more than
 //     twice the best time; then yield heuristic 2 (delta = half and a quarter
-//     of the window); on graphs with out-degree <= 8 the lane-per-vertex
-//     expansion;
+//     of the window);
 //   - group engine (SSSP): a per-group window of 16 and 4 mean weights;
 //   - both: half the batch per launch (query_batch), which keeps a smaller
 //     working set.
@@ -188,17 +187,6 @@ extern "C" fg_status fg_tune_opts_ex(fg_graph *g, int32_t kind, const int32_t *s
           pick = o;
           pick_ms = ms;
         }
-      }
-    }
-    if (pick.group == 1 && g->max_degree <= 8) {
-      fg_opts o = pick;
-      o.threads_per_vertex = 1;
-      st = time_batch(g, kind, src, nq, out.p, nullptr, stream, o, alpha, eps, ea, eb_, &ms);
-      if (st != FG_OK) return st;
-      ++tried;
-      if (ms < pick_ms) {
-        pick = o;
-        pick_ms = ms;
       }
     }
   }
