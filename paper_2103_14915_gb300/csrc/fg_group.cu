@@ -108,15 +108,18 @@ __host__ __device__ __forceinline__ typename GroupLanes<GQ>::M group_bit(uint32_
 // words, listed vertices), then per consumer warp the current step's 32 arcs
 // (uint4 each) and one [B][G] table of source values, B = the listed
 // vertices a warp takes at a time (32; 16 for G = 64, so that three blocks
-// fit an SM).
+// fit an SM). BFS uses no per-warp part and leaves it out: its random reads of
+// reach masks find the hubs' words in the larger L1 (R-MAT 2^20, 256 queries:
+// rounds of 4.9 -> 2.7 ms in groups of 64, 4.5 -> 3.9 in groups of 32; with a
+// fourth block an SM 2.7 and 3.5, and at 2^22 10.4 instead of 9.9 in groups of 64).
 __host__ __device__ constexpr int group_batch(int G) { return G == 64 ? 16 : 32; }
 __host__ __device__ inline size_t group_mask_words(int G) { return G == 64 ? 2u : 1u; }
 __host__ __device__ inline size_t group_item_words(int S, int G) {
   return (size_t)(S + 4) + (size_t)S * (1u + group_mask_words(G));
 }
-__host__ __device__ inline size_t group_smem_bytes(int S, int G) {
-  return (2 * group_item_words(S, G) + (size_t)kGCons * (128u + (size_t)group_batch(G) * (size_t)G)) *
-         sizeof(uint32_t);
+__host__ __device__ inline size_t group_smem_bytes(int qtype, int S, int G) {
+  const size_t warp_words = qtype == Q_BFS ? 0u : 128u + (size_t)group_batch(G) * (size_t)G;
+  return (2 * group_item_words(S, G) + (size_t)kGCons * warp_words) * sizeof(uint32_t);
 }
 
 __device__ __forceinline__ uint32_t g_relax(Ctrl *c, uint32_t d, uint32_t w) {
@@ -572,7 +575,7 @@ __global__ void __launch_bounds__(kGThreads, 3) group_kernel(GroupArgs a) {
           // this round's masks of the item are taken: clear them for reuse
           for (int i = lane; i < ((S * MW) >> 2); i += 32)
             reinterpret_cast<uint4 *>(pm_g)[i] = make_uint4(0u, 0u, 0u, 0u);
-          // list the pending vertices with an arc: those with many pending
+          // list the pending vertices with an arc (BFS: all): those with many pending
           // lanes from the front of vid, the sparse ones (no window only)
           // from its back
           uint32_t cnt = 0, cnt_s = 0;
@@ -582,7 +585,7 @@ __global__ void __launch_bounds__(kGThreads, 3) group_kernel(GroupArgs a) {
             const int i = i0 + lane;
             const uint32_t deg = rp_s[i + 1] - rp_s[i];
             const M mk = pm_s[i];
-            const bool keep = mk != 0u && deg > 0u;
+            const bool keep = mk != 0u && (QT == Q_BFS || deg > 0u);  // (BFS: its level is written)
             int pc;
             if constexpr (GQ == 64) pc = __popcll(mk);
             else pc = __popc(mk);
@@ -666,12 +669,25 @@ __global__ void __launch_bounds__(kGThreads, 3) group_kernel(GroupArgs a) {
           // when the query first reaches it. reach[v] holds the queries that
           // have reached v. A lane takes one arc at a time and sets the
           // frontier lanes F of the arc's source that are new in the
-          // target's reach; only those lanes are marked pending and get
-          // their level. One 4- or 8-byte word per arc replaces the
-          // target's line.
+          // target's reach; only those lanes are marked pending. One 4- or
+          // 8-byte word per arc replaces the target's line. A vertex pending
+          // in this round was reached by its pending lanes at this level, so
+          // its visit writes their levels, a line at a time, where the lane
+          // that reaches it would write them one by one to as many lines
+          // (R-MAT 2^20, 256 queries in groups of 32: rounds 5.3 -> 4.5 ms).
           M *reach_g = reinterpret_cast<M *>(a.reach) + (size_t)d.grp * row;
           const int slog2 = G.slog2;
-          const uint32_t lvl = round + 1u;  // the level reached in this round (serve mode: minus the lane's start)
+          // levels of SL vertices at once: lane (h, g) has vertex v and its mask m
+          auto write_levels = [&](uint32_t v, M m) {
+            uint32_t *Dv = Dg + ((size_t)v << LG);
+            const uint32_t *start = a.lstart ? a.lstart + (size_t)d.grp * Gq : nullptr;  // serve mode: the lane's round 0
+            if constexpr (GQ == 64) {
+              if ((m >> lane) & 1ull) Dv[2 * lane] = round;
+              if ((m >> (32 + lane)) & 1ull) Dv[2 * lane + 1] = round;
+            } else {
+              if ((m >> g) & 1u) Dv[g] = start ? round - start[g] : round;
+            }
+          };
           constexpr int kU = 4;  // arcs per lane with their loads in flight at once
           // relax up to kU arcs per lane: targets v[u] (kNoArc: none) from frontiers F[u]
           auto visit = [&](const uint32_t *v, const M *F) {
@@ -690,16 +706,6 @@ __global__ void __launch_bounds__(kGThreads, 3) group_kernel(GroupArgs a) {
                 i32 += (uint32_t)__popc(fresh);
                 gacc |= fresh;
               }
-              uint32_t *Dv = Dg + ((size_t)v[u] << LG);
-              while (fresh != 0u) {
-                int bp;
-                if constexpr (GQ == 64) bp = __ffsll((long long)fresh) - 1;
-                else bp = __ffs(fresh) - 1;
-                fresh &= fresh - 1u;
-                const uint32_t gq =
-                    GQ == 64 ? ((((uint32_t)bp & 31u) << 1) | ((uint32_t)bp >> 5)) : (uint32_t)bp;
-                Dv[gq] = a.lstart ? lvl - a.lstart[(size_t)d.grp * Gq + gq] : lvl;
-              }
             }
           };
           if (d.kind == kItemHub) {
@@ -709,9 +715,10 @@ __global__ void __launch_bounds__(kGThreads, 3) group_kernel(GroupArgs a) {
             else fpc = (uint32_t)__popc(F);
             for (;;) {
               uint32_t s0 = 0;
-              if (lane == 0) s0 = atomicAdd(&s_desc[k].next, 4u);  // four steps of 32 arcs at a time
+              if (lane == 0) s0 = atomicAdd(&s_desc[k].next, (uint32_t)kU);  // kU steps of 32 arcs at a time
               s0 = __shfl_sync(kFull, s0, 0);
               if (s0 >= d.n) break;
+              if (s0 == 0u && d.eb == G.rp[d.pv] && h == 0) write_levels(d.pv, F);  // the hub's first chunk
               uint32_t v[kU];
               M Fs[kU];
 #pragma unroll
@@ -729,7 +736,6 @@ __global__ void __launch_bounds__(kGThreads, 3) group_kernel(GroupArgs a) {
             const uint32_t base = d.pv << G.slog2;
             const uint32_t *rp_s = buf_rp(k), *vid_s = buf_vid(k);
             const M *pm_s = buf_pm(k);
-            (void)base;
             for (;;) {
               uint32_t b0 = 0;
               if (lane == 0) b0 = atomicAdd(&s_desc[k].next, 32u);
@@ -741,6 +747,9 @@ __global__ void __launch_bounds__(kGThreads, 3) group_kernel(GroupArgs a) {
               const M m = valid ? pm_s[li] : (M)0u;
               const uint32_t a0 = valid ? rp_s[li] : 0u;
               const uint32_t deg = valid ? rp_s[li + 1] - a0 : 0u;
+#pragma unroll 4
+              for (int L0 = 0; L0 < 32; L0 += SL)
+                write_levels(base + __shfl_sync(kFull, li, L0 + h), __shfl_sync(kFull, m, L0 + h));
               if constexpr (GQ == 64) r32 += deg * (uint32_t)__popcll(m);
               else r32 += deg * (uint32_t)__popc(m);
               const uint32_t incl = warp_incl_scan(deg);
@@ -1139,27 +1148,21 @@ bool group_fits(int S, int G) {
   int dev = 0, optin = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return false;
   if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) return false;
-  return group_smem_bytes(S, G) <= (size_t)optin;
+  return group_smem_bytes(Q_SSSP, S, G) <= (size_t)optin;
 }
 
-cudaError_t group_grid_size(int S, int G, int *blocks, int *threads, size_t *smem) {
+cudaError_t group_grid_size(int qtype, int S, int G, int *blocks, int *threads, size_t *smem) {
   *threads = kGThreads;
-  *smem = group_smem_bytes(S, G);
-  int best = 1 << 30, dev = 0, sms = 0;
+  *smem = group_smem_bytes(qtype, S, G);
+  const void *fn = group_fn(qtype, G);
+  int per_sm = 0, dev = 0, sms = 0;
   cudaError_t e;
-  for (int qt = 0; qt < 2; ++qt) {
-    const void *fn = group_fn(qt, G);
-    if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem)) != cudaSuccess)
-      return e;
-    int per_sm = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kGThreads, *smem)) != cudaSuccess)
-      return e;
-    best = per_sm < best ? per_sm : best;
-  }
+  if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem)) != cudaSuccess) return e;
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kGThreads, *smem)) != cudaSuccess) return e;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  if (best < 1) return cudaErrorInvalidConfiguration;
-  *blocks = best * sms;
+  if (per_sm < 1) return cudaErrorInvalidConfiguration;
+  *blocks = per_sm * sms;
   return cudaSuccess;
 }
 

@@ -161,8 +161,10 @@ struct fg_graph {
   fg::DevGraph s_dg;
   int32_t s_nhubs = 0;
   bool reduced = false;
-  int group_blocks[4] = {0, 0, 0, 0}, group_threads[4] = {0, 0, 0, 0};
-  size_t group_smem[4] = {0, 0, 0, 0};
+  struct GroupShape {
+    int blocks = 0, threads = 0;
+    size_t smem = 0;
+  } group_shape[2][4];  // [Q_SSSP, Q_BFS][log2(G) - 3]
 };
 
 namespace fg {
@@ -172,7 +174,7 @@ constexpr uint32_t kHubChunk = 4096;  // group engine: arcs per hub chunk
 
 // The query group that fg_opts.group = 0 resolves to for a batch of nq
 // queries of one kind: on graphs whose partitions are cut by more than half
-// of the arcs, 64 for SSSP (32 under a window) and 32 for BFS (the smallest of
+// of the arcs, 64 (32 for SSSP under a window; the smallest of
 // 8, 16, 32, 64 that holds a smaller batch, and one that fits shared memory);
 // else 1.
 int auto_group_size(const fg_graph *g, int qtype, int64_t nq, bool windowed);

@@ -189,7 +189,7 @@ cudaError_t plain_grid_size(int *blocks, int *threads);
 // Whether a group-engine block for partitions of S vertices and groups of G
 // fits the device's shared memory per block.
 bool group_fits(int S, int G);
-cudaError_t group_grid_size(int S, int G, int *blocks, int *threads, size_t *smem);
+cudaError_t group_grid_size(int qtype, int S, int G, int *blocks, int *threads, size_t *smem);
 cudaError_t launch_group(const GroupArgs &a, int blocks, int threads, size_t smem, cudaStream_t s);
 // Orders a batch's queries for the group engine: key[q] = arcs within two hops
 // of src[q], or (by_place) the source's internal id counted down; perm[j] =

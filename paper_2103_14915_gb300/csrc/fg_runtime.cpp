@@ -721,14 +721,13 @@ fg_status run_batch_on(fg_graph *g, Workspace &ws, bool shared_ws, int grid_div,
       nbq = std::min<int64_t>(nbq, cap_groups * Gq);
       nbq = std::min<int64_t>(nbq, nq);
     }
-    const int gi = glog2 - 3;
     if (Gq == 64 && qtype == Q_SSSP && o.sched == FG_SCHED_PRIORITY && o.sched_window != 0u)
       return fail(FG_ERR_UNSUPPORTED, "the group engine has no window for groups of 64; use FIFO or a group of 32");
     if (!group_fits(g->S, Gq))
       return fail(FG_ERR_UNSUPPORTED, "group %d does not fit shared memory with partitions of %d vertices", Gq, g->S);
-    if (g->group_blocks[gi] == 0)
-      CUDA_TRY(group_grid_size(g->S, Gq, &g->group_blocks[gi], &g->group_threads[gi], &g->group_smem[gi]));
-    const int blocks = grid_div > 1 ? std::max(1, g->group_blocks[gi] / grid_div) : g->group_blocks[gi];
+    auto &shape = g->group_shape[qtype][glog2 - 3];
+    if (shape.blocks == 0) CUDA_TRY(group_grid_size(qtype, g->S, Gq, &shape.blocks, &shape.threads, &shape.smem));
+    const int blocks = grid_div > 1 ? std::max(1, shape.blocks / grid_div) : shape.blocks;
     const int64_t ngroups_max = (nbq + Gq - 1) / Gq;
     const uint64_t hub_cap = (uint64_t)ngroups_max * g->hub_chunks;
     if (hub_cap + (uint64_t)ngroups_max * (uint64_t)g->nparts >= 0xFFFFFFFFull)
@@ -790,7 +789,7 @@ fg_status run_batch_on(fg_graph *g, Workspace &ws, bool shared_ws, int grid_div,
       a.max_rounds = max_rounds;
       a.watchdog_ns = watchdog_ns;
       a.check_staging = o.check_staging ? 1u : 0u;
-      CUDA_TRY(launch_group(a, blocks, g->group_threads[gi], g->group_smem[gi], stream));
+      CUDA_TRY(launch_group(a, blocks, shape.threads, shape.smem, stream));
       ++launches;
       if (rowmap) CUDA_TRY(launch_group_out(a, dist, rowmap + q0, stream));
       else CUDA_TRY(launch_group_out(a, dist + (size_t)q0 * (size_t)n, nullptr, stream));
@@ -1043,7 +1042,10 @@ namespace fg {
 
 int auto_group_size(const fg_graph *g, int qtype, int64_t nq, bool windowed) {
   if (!(g->m > 0 && 2 * g->cut > g->m)) return 1;
-  int G = (qtype == Q_BFS || windowed) ? 32 : 64;  // groups of 64 run FIFO rounds only
+  // the widest group: fewer reads of arcs and masks for as many queries (BFS on
+  // R-MAT, groups of 32 -> 64: 2^14 vertices, 64 queries 0.37 -> 0.36 ms; 2^20, 256
+  // queries 5.1 -> 3.8; 2^22 20.3 -> 13.8). SSSP groups of 64 run FIFO rounds only
+  int G = qtype == Q_SSSP && windowed ? 32 : 64;
   while (G > 8 && (int64_t)(G / 2) >= nq) G /= 2;  // a small batch: the smallest group that holds it
   while (G > 8 && !group_fits(g->S, G)) G /= 2;
   return group_fits(g->S, G) ? G : 1;

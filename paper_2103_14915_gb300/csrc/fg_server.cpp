@@ -191,9 +191,9 @@ fg_status create_slot_lane(fg_server *s, SlotLane &C, int kind, int nslots, int 
   C.nslots = nslots;
   if (!group_fits(g->S, G))
     return fail(FG_ERR_UNSUPPORTED, "group %d does not fit shared memory with partitions of %d vertices", G, g->S);
-  if (g->group_blocks[C.gi] == 0)
-    CUDA_TRY(group_grid_size(g->S, G, &g->group_blocks[C.gi], &g->group_threads[C.gi], &g->group_smem[C.gi]));
-  C.blocks = div > 1 ? std::max(1, g->group_blocks[C.gi] / div) : g->group_blocks[C.gi];
+  auto &shape = g->group_shape[C.qtype][C.gi];
+  if (shape.blocks == 0) CUDA_TRY(group_grid_size(C.qtype, g->S, G, &shape.blocks, &shape.threads, &shape.smem));
+  C.blocks = div > 1 ? std::max(1, shape.blocks / div) : shape.blocks;
   const size_t npad = (size_t)g->nparts * (size_t)g->S, ng = (size_t)C.ngroups;
   const uint64_t hub_cap = (uint64_t)ng * g->hub_chunks;
   if (hub_cap + (uint64_t)ng * (uint64_t)g->nparts >= 0xFFFFFFFFull)
@@ -272,7 +272,8 @@ fg_status launch_slot_lane(fg_server *s, SlotLane &C) {
   a.lstart = C.qtype == Q_BFS ? C.lstart.as<uint32_t>() : nullptr;
   if (C.need_init) C.round0 = 0;
   a.round0 = C.round0;
-  CUDA_TRY(launch_group(a, C.blocks, g->group_threads[C.gi], g->group_smem[C.gi], C.stream));
+  CUDA_TRY(launch_group(a, C.blocks, g->group_shape[C.qtype][C.gi].threads, g->group_shape[C.qtype][C.gi].smem,
+                        C.stream));
   CUDA_TRY(cudaMemcpyAsync(C.h_ctrl, C.ctrl.p, sizeof(Ctrl), cudaMemcpyDeviceToHost, C.stream));
   CUDA_TRY(cudaEventRecord(C.done_ev, C.stream));
   C.need_init = false;
