@@ -1045,33 +1045,51 @@ done:
 }
 
 // D[group][v][g] (internal order) -> out[row(group * G + g)][orig(v)] for v < n,
-// row(j) = rowmap[j] (or j without a map). A block moves 32 vertices of one
-// group: 32 * G words read as whole lines, transposed in shared memory,
-// written as G runs of 32 values. Where arcs were left out, the values are
-// held against the overflow limit on the way.
+// row(j) = rowmap[j] (or j without a map). A block moves kOutV vertices of one
+// group: their lines are read 16 bytes a lane, transposed in shared memory and
+// written as G runs of kOutV values. Both sides are touched once, so they go
+// past the caches' keep lists. HBM bounds it: OUT_NOTE. Where arcs were left
+// out, the values are held against the overflow limit on the way.
+constexpr int kOutV = 64;
+
+template <int G>
 __global__ void __launch_bounds__(256) group_out_kernel(GroupArgs a, uint32_t *out, const int32_t *rowmap,
                                                         int64_t tiles_per_group) {
-  __shared__ uint32_t t[64][33];
-  const int32_t G = a.G;
+  __shared__ uint32_t t[G][kOutV + 1];
+  constexpr int kQ4 = G / 4;                     // 16-byte pieces of a line
+  constexpr int kPer = (kOutV * kQ4 + 255) / 256;  // pieces a thread
   const int64_t n = a.g.n;
   const int64_t grp = blockIdx.x / tiles_per_group;
-  const int64_t v0 = (blockIdx.x % tiles_per_group) * 32;
+  const int64_t v0 = (blockIdx.x % tiles_per_group) * kOutV;
   const uint32_t lim = overflow_limit(a.g);
-  const uint32_t *src = a.D + ((size_t)grp * (size_t)a.npad + (size_t)v0) * (size_t)G;
-  for (int i = threadIdx.x; i < 32 * G; i += blockDim.x) {
-    const int vl = i >> a.glog2, gq = i & (G - 1);
-    const uint32_t x = v0 + vl < n ? src[i] : kInf;
-    t[gq][vl] = x;
-    if (a.all_rp != nullptr) check_all_arcs(a, lim, (uint32_t)(v0 + vl), x);
+  const uint4 *src = reinterpret_cast<const uint4 *>(a.D + ((size_t)grp * (size_t)a.npad + (size_t)v0) * (size_t)G);
+  uint4 x[kPer];
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+    const int i = k * 256 + (int)threadIdx.x;
+    if (i < kOutV * kQ4 && v0 + i / kQ4 < n) x[k] = __ldcs(src + i);
+  }
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+    const int i = k * 256 + (int)threadIdx.x, vl = i / kQ4, q = (i % kQ4) * 4;
+    if (i < kOutV * kQ4 && v0 + vl < n) {
+      const uint32_t y[4] = {x[k].x, x[k].y, x[k].z, x[k].w};
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        t[q + c][vl] = y[c];
+        if (a.all_rp != nullptr) check_all_arcs(a, lim, (uint32_t)(v0 + vl), y[c]);
+      }
+    }
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < 32 * G; i += blockDim.x) {
-    const int gq = i >> 5, vl = i & 31;
+#pragma unroll
+  for (int k = 0; k < kOutV * G / 256; ++k) {
+    const int i = k * 256 + (int)threadIdx.x, gq = i / kOutV, vl = i % kOutV;
     const int64_t q = grp * G + gq, v = v0 + vl;
     if (q < a.nq && v < n) {
       const int64_t o = a.g.orig ? (int64_t)a.g.orig[v] : v;
       const int64_t r = rowmap ? (int64_t)rowmap[q] : q;
-      out[r * n + o] = t[gq][vl];
+      __stcs(out + r * n + o, t[gq][vl]);
     }
   }
 }
@@ -1173,11 +1191,14 @@ cudaError_t launch_group(const GroupArgs &a, int blocks, int threads, size_t sme
 }
 
 cudaError_t launch_group_out(const GroupArgs &a, uint32_t *out, const int32_t *rowmap, cudaStream_t s) {
-  const int64_t n = a.g.n;
-  const int64_t tiles = (n + 31) / 32;
+  const int64_t tiles = ((int64_t)a.g.n + kOutV - 1) / kOutV;
   const int64_t grid = tiles * (int64_t)a.ngroups;
   if (grid <= 0) return cudaSuccess;
-  group_out_kernel<<<(unsigned)grid, 256, 0, s>>>(a, out, rowmap, tiles);
+  const dim3 gr((unsigned)grid), bl(256);
+  if (a.G == 8) group_out_kernel<8><<<gr, bl, 0, s>>>(a, out, rowmap, tiles);
+  else if (a.G == 16) group_out_kernel<16><<<gr, bl, 0, s>>>(a, out, rowmap, tiles);
+  else if (a.G == 32) group_out_kernel<32><<<gr, bl, 0, s>>>(a, out, rowmap, tiles);
+  else group_out_kernel<64><<<gr, bl, 0, s>>>(a, out, rowmap, tiles);
   return cudaGetLastError();
 }
 
