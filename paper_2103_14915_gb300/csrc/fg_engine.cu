@@ -1402,11 +1402,24 @@ static const void *engine_fn(int qtype, bool pairs) {
   }
 }
 
+// Lets a kernel be launched with any dynamic shared memory the device has: the
+// limit belongs to the kernel, not to a graph, and graphs of different
+// partition sizes are in use at once.
+cudaError_t allow_dynamic_smem(const void *fn) {
+  cudaFuncAttributes at;
+  int dev = 0, optin = 0;
+  cudaError_t e = cudaFuncGetAttributes(&at, fn);
+  if (e == cudaSuccess) e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)at.sharedSizeBytes);
+}
+
 cudaError_t engine_grid_size(int qtype, bool pairs, int S, int *blocks, int *threads, size_t *smem) {
   const void *fn = engine_fn(qtype, pairs);
   *threads = kThreads;
   *smem = (size_t)kWarps * warp_smem_words(qtype == Q_PPR, S) * sizeof(uint32_t);
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem);
+  cudaError_t e = allow_dynamic_smem(fn);
   if (e != cudaSuccess) return e;
   int per_sm = 0, dev = 0, sms = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kThreads, *smem);

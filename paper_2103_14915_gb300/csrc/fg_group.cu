@@ -1176,7 +1176,7 @@ cudaError_t group_grid_size(int qtype, int S, int G, int *blocks, int *threads, 
   const void *fn = group_fn(qtype, G);
   int per_sm = 0, dev = 0, sms = 0;
   cudaError_t e;
-  if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem)) != cudaSuccess) return e;
+  if ((e = allow_dynamic_smem(fn)) != cudaSuccess) return e;
   if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kGThreads, *smem)) != cudaSuccess) return e;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;

@@ -151,7 +151,7 @@ struct fg_graph {
   int plain_blocks = 0, plain_threads = 0;
   // group engine: the hubs, vertices with more than kHubMin arcs (internal ids),
   // relaxed in chunks of at most kHubChunk arcs spread over blocks, and the
-  // number of chunks they make; launch shapes per group size (index log2(G) - 3)
+  // number of chunks they make; launch shapes below
   fg::DevBuf hubs;
   int32_t nhubs = 0;
   uint64_t hub_chunks = 0;
@@ -161,10 +161,10 @@ struct fg_graph {
   fg::DevGraph s_dg;
   int32_t s_nhubs = 0;
   bool reduced = false;
-  struct GroupShape {
+  struct group_shape_t {
     int blocks = 0, threads = 0;
     size_t smem = 0;
-  } group_shape[2][4];  // [Q_SSSP, Q_BFS][log2(G) - 3]
+  } group_shape[2][4][8];  // [Q_SSSP, Q_BFS][log2(G) - 3][log2(S) - 5]
 };
 
 namespace fg {

@@ -179,6 +179,7 @@ struct PlainArgs {
 };
 
 // kernel launchers (fg_engine.cu / fg_plain.cu); return the CUDA error of the launch
+cudaError_t allow_dynamic_smem(const void *fn);
 cudaError_t engine_grid_size(int qtype, bool pairs, int S, int *blocks, int *threads, size_t *smem);
 cudaError_t launch_engine(const EngineArgs &a, int blocks, int threads, size_t smem, cudaStream_t s);
 cudaError_t launch_pair_records(const DevGraph &g, uint2 *out, cudaStream_t s);

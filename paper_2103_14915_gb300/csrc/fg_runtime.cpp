@@ -591,6 +591,34 @@ fg_status ensure_plain_ws(fg_graph *g, Workspace &ws, int qtype, int64_t nb, boo
 
 namespace fg {
 
+// The partitions a group-engine batch of ngroups groups runs on, and its
+// launch shape. A work item is one (partition, group), taken by one block, and
+// its vertices go through the block's eight warps 16 or 32 at a time, so a
+// round lasts as long as the longest chain of items on a block. With fewer
+// than kItemsPerBlock items a block when every item is pending, the graph's
+// partitions are cut into halves until there are as many (the vertex order
+// stays; not below kMinSplit vertices). R-MAT, SSSP in groups of 64, S = 1024
+// against the cut ones (GB300): 2^14 vertices, 64 queries 1.69 -> 1.15 ms; 2^18,
+// 256 queries 3.57 -> 3.15; 2^20, 64 queries 3.14 -> 2.74 (256 queries have 4,096
+// items: 7.50, and 7.46 cut once, 8.60 twice).
+constexpr int64_t kItemsPerBlock = 4;
+constexpr int kMinSplit = 64;
+
+static fg_status group_partitions(fg_graph *g, int qtype, int glog2, int64_t ngroups, DevGraph *gg,
+                                  const fg_graph::group_shape_t **shape_out) {
+  *gg = g->dg;
+  for (;;) {
+    fg_graph::group_shape_t &shape = g->group_shape[qtype][glog2 - 3][gg->slog2 - 5];
+    if (shape.blocks == 0)
+      CUDA_TRY(group_grid_size(qtype, gg->S, 1 << glog2, &shape.blocks, &shape.threads, &shape.smem));
+    *shape_out = &shape;
+    if (gg->S <= kMinSplit || (int64_t)gg->nparts * ngroups >= kItemsPerBlock * shape.blocks) return FG_OK;
+    gg->S /= 2;
+    gg->slog2 -= 1;
+    gg->nparts = (int32_t)(((int64_t)gg->n + gg->S - 1) / gg->S);
+  }
+}
+
 // One batch on workspace ws. shared_ws: ws is the graph's own workspace, so
 // the batch waits for the graph's previous batch (stream order across
 // streams). grid_div > 1 launches the engine on 1/grid_div of the resident
@@ -701,7 +729,6 @@ fg_status run_batch_on(fg_graph *g, Workspace &ws, bool shared_ws, int grid_div,
   if (o.mode == FG_MODE_BUFFERED && Gq > 1) {
     int glog2 = 0;
     while ((1 << glog2) < Gq) ++glog2;
-    const int64_t npad = (int64_t)g->nparts * (int64_t)g->S;
     // queries per launch from the device's free memory: per group the state
     // (G values per vertex), two pending masks per vertex, the dirty flags and
     // work items of its partitions and its hub chunks
@@ -713,7 +740,8 @@ fg_status run_batch_on(fg_graph *g, Workspace &ws, bool shared_ws, int grid_div,
                           ws.g_reach.bytes;
       const double avail = 0.9 * (double)(free_b + held) - 512.0 * 1024 * 1024;
       const double mask_b = Gq == 64 ? 8.0 : 4.0;
-      const double per_group = (double)npad * 4.0 * (double)Gq + (qtype == Q_BFS ? 3.0 : 2.0) * mask_b * (double)npad +
+      const double npad = (double)g->nparts * (double)g->S;
+      const double per_group = npad * 4.0 * (double)Gq + (qtype == Q_BFS ? 3.0 : 2.0) * mask_b * npad +
                                24.0 * (double)g->nparts + 20.0 * (double)g->hub_chunks + 8.0;
       int64_t cap_groups = std::max<int64_t>(1, (int64_t)(avail / per_group));
       const int64_t key_cap = (int64_t)(0xFFFFFFF0ull / (uint64_t)g->nparts);
@@ -725,19 +753,24 @@ fg_status run_batch_on(fg_graph *g, Workspace &ws, bool shared_ws, int grid_div,
       return fail(FG_ERR_UNSUPPORTED, "the group engine has no window for groups of 64; use FIFO or a group of 32");
     if (!group_fits(g->S, Gq))
       return fail(FG_ERR_UNSUPPORTED, "group %d does not fit shared memory with partitions of %d vertices", Gq, g->S);
-    auto &shape = g->group_shape[qtype][glog2 - 3];
-    if (shape.blocks == 0) CUDA_TRY(group_grid_size(qtype, g->S, Gq, &shape.blocks, &shape.threads, &shape.smem));
-    const int blocks = grid_div > 1 ? std::max(1, shape.blocks / grid_div) : shape.blocks;
     const int64_t ngroups_max = (nbq + Gq - 1) / Gq;
+    DevGraph gg;  // the partitions of this batch
+    const fg_graph::group_shape_t *shape = nullptr;
+    {
+      const fg_status st = group_partitions(g, qtype, glog2, ngroups_max, &gg, &shape);
+      if (st != FG_OK) return st;
+    }
+    const int64_t nparts = gg.nparts, npad = nparts * (int64_t)gg.S;
+    const int blocks = grid_div > 1 ? std::max(1, shape->blocks / grid_div) : shape->blocks;
     const uint64_t hub_cap = (uint64_t)ngroups_max * g->hub_chunks;
-    if (hub_cap + (uint64_t)ngroups_max * (uint64_t)g->nparts >= 0xFFFFFFFFull)
+    if (hub_cap + (uint64_t)ngroups_max * (uint64_t)nparts >= 0xFFFFFFFFull)
       return fail(FG_ERR_UNSUPPORTED, "too many work items for one launch; lower query_batch");
     CUDA_TRY(ws.g_D.reserve(4 * (size_t)ngroups_max * (size_t)npad * (size_t)Gq));
     CUDA_TRY(ws.g_pend.reserve((Gq == 64 ? 16 : 8) * (size_t)ngroups_max * (size_t)npad));
     if (qtype == Q_BFS) CUDA_TRY(ws.g_reach.reserve((Gq == 64 ? 8 : 4) * (size_t)ngroups_max * (size_t)npad));
-    CUDA_TRY(ws.g_dirty.reserve(8 * (size_t)ngroups_max * (size_t)g->nparts));
+    CUDA_TRY(ws.g_dirty.reserve(8 * (size_t)ngroups_max * (size_t)nparts));
     // work items, then (G = 64) the upper mask words of the hub-chunk items
-    CUDA_TRY(ws.g_items.reserve(16 * (size_t)(hub_cap + (uint64_t)ngroups_max * (uint64_t)g->nparts) +
+    CUDA_TRY(ws.g_items.reserve(16 * (size_t)(hub_cap + (uint64_t)ngroups_max * (uint64_t)nparts) +
                                 (Gq == 64 ? 4 * (size_t)hub_cap : 0)));
     CUDA_TRY(ws.g_best.reserve(8 * (size_t)ngroups_max));
     CUDA_TRY(ws.ctrl.reserve(sizeof(Ctrl)));
@@ -767,6 +800,9 @@ fg_status run_batch_on(fg_graph *g, Workspace &ws, bool shared_ws, int grid_div,
       const int64_t cnt_q = std::min<int64_t>(nbq, nq - q0);
       GroupArgs a;
       set_group_graph(g, qtype, a);
+      a.g.S = gg.S;
+      a.g.slog2 = gg.slog2;
+      a.g.nparts = gg.nparts;
       a.qtype = qtype;
       a.nq = (int32_t)cnt_q;
       a.G = Gq;
@@ -779,7 +815,7 @@ fg_status run_batch_on(fg_graph *g, Workspace &ws, bool shared_ws, int grid_div,
       a.dirty = ws.g_dirty.as<uint32_t>();
       a.items = ws.g_items.as<uint4>();
       a.hub_cap = (uint32_t)((uint64_t)a.ngroups * g->hub_chunks);
-      a.hub_hi = Gq == 64 ? reinterpret_cast<uint32_t *>(a.items + a.hub_cap + (size_t)a.ngroups * (size_t)g->nparts)
+      a.hub_hi = Gq == 64 ? reinterpret_cast<uint32_t *>(a.items + a.hub_cap + (size_t)a.ngroups * (size_t)nparts)
                           : nullptr;
       a.hub_chunk = kHubChunk;
       a.window = qtype == Q_SSSP && o.sched == FG_SCHED_PRIORITY ? o.sched_window : 0u;
@@ -789,7 +825,7 @@ fg_status run_batch_on(fg_graph *g, Workspace &ws, bool shared_ws, int grid_div,
       a.max_rounds = max_rounds;
       a.watchdog_ns = watchdog_ns;
       a.check_staging = o.check_staging ? 1u : 0u;
-      CUDA_TRY(launch_group(a, blocks, shape.threads, shape.smem, stream));
+      CUDA_TRY(launch_group(a, blocks, shape->threads, shape->smem, stream));
       ++launches;
       if (rowmap) CUDA_TRY(launch_group_out(a, dist, rowmap + q0, stream));
       else CUDA_TRY(launch_group_out(a, dist + (size_t)q0 * (size_t)n, nullptr, stream));

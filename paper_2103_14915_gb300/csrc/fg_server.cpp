@@ -191,7 +191,7 @@ fg_status create_slot_lane(fg_server *s, SlotLane &C, int kind, int nslots, int 
   C.nslots = nslots;
   if (!group_fits(g->S, G))
     return fail(FG_ERR_UNSUPPORTED, "group %d does not fit shared memory with partitions of %d vertices", G, g->S);
-  auto &shape = g->group_shape[C.qtype][C.gi];
+  auto &shape = g->group_shape[C.qtype][C.gi][g->slog2 - 5];
   if (shape.blocks == 0) CUDA_TRY(group_grid_size(C.qtype, g->S, G, &shape.blocks, &shape.threads, &shape.smem));
   C.blocks = div > 1 ? std::max(1, shape.blocks / div) : shape.blocks;
   const size_t npad = (size_t)g->nparts * (size_t)g->S, ng = (size_t)C.ngroups;
@@ -272,8 +272,8 @@ fg_status launch_slot_lane(fg_server *s, SlotLane &C) {
   a.lstart = C.qtype == Q_BFS ? C.lstart.as<uint32_t>() : nullptr;
   if (C.need_init) C.round0 = 0;
   a.round0 = C.round0;
-  CUDA_TRY(launch_group(a, C.blocks, g->group_shape[C.qtype][C.gi].threads, g->group_shape[C.qtype][C.gi].smem,
-                        C.stream));
+  CUDA_TRY(launch_group(a, C.blocks, g->group_shape[C.qtype][C.gi][g->slog2 - 5].threads,
+                        g->group_shape[C.qtype][C.gi][g->slog2 - 5].smem, C.stream));
   CUDA_TRY(cudaMemcpyAsync(C.h_ctrl, C.ctrl.p, sizeof(Ctrl), cudaMemcpyDeviceToHost, C.stream));
   CUDA_TRY(cudaEventRecord(C.done_ev, C.stream));
   C.need_init = false;
