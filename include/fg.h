@@ -116,9 +116,11 @@ typedef struct {
                                every arc leaves its partition: power-law graphs); 1 = one query
                                per warp and visit (best on road-like graphs, whose partitions
                                keep most arcs inside). 0 (default) = automatic: when more than
-                               half of the graph's arcs cross partitions, 64 (32 for SSSP with a
+                               half of the graph's arcs cross partitions, or it has out-degrees
+                               above 64 and at most 16 partitions, 64 (32 for SSSP with a
                                sched_window; a smaller batch takes the smallest group that
-                               holds it), else 1. PPR
+                               holds it, and for SSSP with n * nq of at most 2^22, 8 up to 32
+                               queries and 16 up to 64), else 1. PPR
                                always runs one query per warp. In the group engine, sched_window
                                (SSSP) bounds each round to values below the group's smallest
                                pending value plus the window (groups of 8 to 32 only: a group of
@@ -183,8 +185,8 @@ void fg_default_graph_opts(fg_graph_opts *o);
  * arrays are copied; the caller keeps ownership. Requires 1 <= n < 2^31 and
  * m < 2^32. Partitions the vertices (Def. 2.1) and stores the graph
  * partition-major on the device. Synchronous. *out receives the handle.
- * A weighted graph of at least 65,536 arcs, more than half of them between
- * partitions, also gets a second copy without the arcs that lie on no shortest
+ * A weighted graph of at least 32,768 arcs on which the group engine is the
+ * automatic choice also gets a second copy without the arcs that lie on no shortest
  * path, if enough are found: SSSP in the group engine runs on that copy, with
  * the same distances (16 * n words of device memory during the call).
  */

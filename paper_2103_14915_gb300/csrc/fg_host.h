@@ -172,11 +172,13 @@ namespace fg {
 constexpr uint32_t kHubMin = 512;     // group engine: vertices with more arcs are hubs
 constexpr uint32_t kHubChunk = 4096;  // group engine: arcs per hub chunk
 
-// The query group that fg_opts.group = 0 resolves to for a batch of nq
-// queries of one kind: on graphs whose partitions are cut by more than half
-// of the arcs, 64 (32 for SSSP under a window; the smallest of
-// 8, 16, 32, 64 that holds a smaller batch, and one that fits shared memory);
-// else 1.
+// Whether the group engine is the automatic choice on a graph.
+bool groups_by_default(const fg_graph *g);
+
+// The query group that fg_opts.group = 0 resolves to for a batch of nq queries
+// of one kind: where groups_by_default, 64, or 32 for SSSP under a window, or 8
+// or 16 for SSSP with little state (the smallest of 8, 16, 32, 64 that holds a
+// smaller batch, and one that fits shared memory); else 1.
 int auto_group_size(const fg_graph *g, int qtype, int64_t nq, bool windowed);
 
 // The graph and hubs a group-engine launch of this query kind runs on.

@@ -143,14 +143,16 @@ static void release_reduced(fg_graph *g) {
 // fg_reduce.cu shows to lie on no shortest path. Built where the group engine
 // is the automatic choice and an arc can be beaten at all (a walk of two arcs
 // is at least twice the smallest weight), for graphs of at least kReduceMinArcs
-// arcs, and kept when it leaves at most 3/4 of them. Without memory for it the
+// arcs (below, the millisecond it takes once is what it saves in a batch or two;
+// R-MAT of 45,000 arcs, 64 queries in groups of 8: 1.21 ms a batch with every arc,
+// 0.43 without), and kept when it leaves at most 3/4 of them. Without memory for it the
 // graph does without. Other CUDA errors are returned.
-constexpr int64_t kReduceMinArcs = 1 << 16;
+constexpr int64_t kReduceMinArcs = 1 << 15;
 
 static cudaError_t build_reduced(fg_graph *g, const std::vector<uint32_t> &rp, const std::vector<uint32_t> &adj,
                                  const std::vector<uint32_t> &wt) {
   const int64_t n = g->n, m = g->m;
-  if (m < kReduceMinArcs || 2 * g->cut <= m) return cudaSuccess;
+  if (m < kReduceMinArcs || !groups_by_default(g)) return cudaSuccess;
   if (2 * (uint64_t)g->min_weight >= (uint64_t)g->max_weight) return cudaSuccess;
   // the vertices of largest out-degree, ties by smaller id
   HubSet hubs;
@@ -788,7 +790,7 @@ fg_status run_batch_on(fg_graph *g, Workspace &ws, bool shared_ws, int grid_div,
       CUDA_TRY(ws.g_psrc.reserve(4 * (size_t)nq));
       // graphs whose partitions keep most arcs inside (road-like): nearby
       // sources together; else sources of alike reach together
-      const bool by_place = !(g->m > 0 && 2 * g->cut > g->m);
+      const bool by_place = !groups_by_default(g);
       CUDA_TRY(launch_group_order(g->dg, src, (int32_t)nq, by_place, ws.g_key.as<unsigned long long>(),
                                   ws.g_perm.as<int32_t>(),
                                   ws.g_psrc.as<int32_t>(), stream));
@@ -1076,12 +1078,33 @@ extern "C" fg_status fg_sync(void *stream_v) {
 
 namespace fg {
 
+// Whether the group engine is the automatic choice on a graph: more than half
+// of its arcs cross partitions, or it has hubs (more arcs than any road
+// crossing) and so few partitions that growing them keeps arcs inside whatever
+// the graph. R-MAT of 2,048 and 4,096 vertices (2 and 4 partitions, 12 and 35 % of
+// the arcs cut), SSSP with 64 queries: 4.8 and 12.7 ms one query per warp, 0.43
+// and 0.49 in groups; BFS 1.6 and 4.6 against 0.25 and 0.27 (GB300).
+bool groups_by_default(const fg_graph *g) {
+  constexpr uint32_t kRoadDegree = 64;
+  constexpr int kFewPartitions = 16;
+  return g->m > 0 && (2 * g->cut > g->m || (g->max_degree > kRoadDegree && g->nparts <= kFewPartitions));
+}
+
+constexpr int64_t kSmallState = 1 << 22;  // values (16 MB)
+
 int auto_group_size(const fg_graph *g, int qtype, int64_t nq, bool windowed) {
-  if (!(g->m > 0 && 2 * g->cut > g->m)) return 1;
+  if (!groups_by_default(g)) return 1;
   // the widest group: fewer reads of arcs and masks for as many queries (BFS on
   // R-MAT, groups of 32 -> 64: 2^14 vertices, 64 queries 0.37 -> 0.36 ms; 2^20, 256
   // queries 5.1 -> 3.8; 2^22 20.3 -> 13.8). SSSP groups of 64 run FIFO rounds only
   int G = qtype == Q_SSSP && windowed ? 32 : 64;
+  // SSSP with little state is bound by the chain of a vertex's line and arcs, not
+  // by what it reads: groups of 8 or 16, whose warps take four or two arcs at once,
+  // as long as that makes at most four groups (2^12, 2^14 and 2^16 vertices: 13
+  // queries 0.61, 0.77, 0.77 ms in one group of 16, 0.43, 0.54, 0.61 in groups of 8; 64
+  // queries 0.74, 1.15, 1.21 in one group of 64, 0.71, 0.97, 1.23 in groups of 16; 2^18,
+  // 13 queries 1.09 and 0.88)
+  if (qtype == Q_SSSP && g->n * nq <= kSmallState && nq <= 64) G = nq <= 32 ? 8 : 16;
   while (G > 8 && (int64_t)(G / 2) >= nq) G /= 2;  // a small batch: the smallest group that holds it
   while (G > 8 && !group_fits(g->S, G)) G /= 2;
   return group_fits(g->S, G) ? G : 1;

@@ -57,7 +57,7 @@ CASES = {
     "zero": (lambda: multigraph(70001, 0, 9), True),
     "last_word_full": (lambda: multigraph(65536, 1, 100), True),
     "last_word_of_one": (lambda: multigraph(65537, 1, 100), True),
-    "too_few_arcs": (lambda: multigraph(65535, 1, 100), False),
+    "too_few_arcs": (lambda: multigraph(32767, 1, 100), False),
     "no_arc_can_be_beaten": (lambda: inputs.rmat(12, 16, seed=6, weights=(128, 256)), False),
 }
 
