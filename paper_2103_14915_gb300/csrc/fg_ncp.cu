@@ -8,34 +8,38 @@
 // vol = sum of out-degrees, cut = arcs from S_k to the rest; and, across all
 // queries of the call, the profile NCP(k) = min over queries of phi(S_k).
 //
-// One block per query (with few queries, several blocks per query, below):
-//   1. select  one pass over the row: vertex v gets the 64-bit sort key
-//              (~key bits << 32 | v), unique, ascending = key descending then
-//              id ascending; keys that may still be among the `top` smallest
-//              go into a shared-memory buffer, which is cut back to exactly
-//              `top` keys (radix select over 8-bit digits inside the buffer)
-//              whenever the next tile might not fit, after which only keys
-//              below the `top`-th are admitted. With the tiles in a scrambled
-//              order about top * (1 + ln(#positive / top)) keys are admitted;
-//              a vertex whose key must round below the threshold is skipped
-//              before the division (an FP32 test with a stated bound);
-//   2. sort    bitonic sort of the kept keys;
-//   3. rank    a shared-memory hash from each chosen vertex's internal id to
-//              its sweep rank; the neighbours ranked before a vertex are
-//              counted by one lane (light vertex), one warp (medium) or the
-//              whole block (a hub of more than 4,096 arcs);
-//   4. scan    prefix sums of d(v) - 2 * inside(v) and of d(v) give cut and vol
-//              exactly in int64; phi = cut / den in FP64.
-// When there are too few rows to give every SM two blocks, each row is split
-// into segments: a block per segment runs step 1 and leaves its top keys in
-// scratch (from the stream-ordered allocator), and a block per row merges the
-// segments' keys through the same buffer and runs steps 2-4. The kept set
-// does not depend on the split.
-//
-// The row read (p from HBM, 4 B per vertex, float4 loads one tile ahead; the
-// degree table, shared by all queries, mostly from L2) is the traffic; steps
-// 2-4 touch only shared memory and the chosen vertices' adjacency.
+// The sort key of a vertex is 64 bits (~key bits << 32 | id), unique, ascending =
+// key descending then id ascending. Five kernels, each spread over as many
+// blocks as its work has room for:
+//   sample   a histogram over 4,096 bins of the key bits (exponent and four
+//            bits of mantissa) of one row chunk in sixteen (of all chunks up to
+//            2^16 vertices), and from it a bin edge that the `top`-th key lies
+//            above for all but certain, with about 1.4 times as many keys above
+//            it as are wanted;
+//   filter   one pass over the row: the sort keys of the vertices at or above the
+//            edge go to the row's list, and the vertices with p > 0 are counted.
+//            A vertex whose key must round below the edge is skipped before the
+//            division (an FP32 test with a stated bound);
+//   order    a block per row sorts the list and keeps the first `top`. A row whose
+//            list is too long, or shorter than it has to be (the sample says
+//            nothing about the rows of an adversary, or about ties), is streamed
+//            instead through a buffer in shared memory that is cut back to the
+//            `top` smallest keys whenever it fills: the kept set is the same;
+//   inside   the neighbours ranked before each kept vertex: a shared-memory hash
+//            from internal id to rank, the arcs of a block's vertices spread
+//            evenly over its threads;
+//   scan     prefix sums of d(v) - 2 * inside(v) and of d(v) give cut and vol
+//            exactly in int64; phi = cut / den in FP64.
+// The row read (p from HBM, 4 B per vertex; the degree table, shared by all
+// queries, mostly from L2) is the traffic and bounds the filter; the others work
+// on shared memory and the kept vertices' adjacency. R-MAT 2^20, 105 rows, top
+// 4,096 (GB300): sample 16 us, edge 4, filter 116 (440 MB at 3.8 TB/s, and as
+// much again of degrees from L2), order 55, inside 100, scan 18, and 0.33 ms for
+// the call. One block per row doing all of it took 1.94 ms: 105 blocks leave a
+// third of the SMs idle, and the threshold that its buffer finds on the way lets
+// five times as many keys in. Rows of few vertices take one block (below).
 #include <algorithm>
+#include <cmath>
 #include <cstdint>
 #include <cstdio>
 #include <mutex>
@@ -53,18 +57,11 @@ constexpr int kHash = 2 * kMaxTop;              // hash slots (load <= 1/2)
 constexpr int kHashLog2 = 13;
 constexpr uint32_t kEmpty = 0xFFFFFFFFu;
 static_assert(kHash == (1 << kHashLog2), "hash size");
-static_assert(kCap * 8 == kHash * 8, "the hash reuses the candidate buffer");
 
-// dynamic shared memory
-//   A: cand[kCap] u64 (steps 1-2), then hash keys[kHash] u32 + vals[kHash] u32 (step 3)
-//   B + C: the cut-back copy tmp[kMaxTop] u64 (step 1); then
-//   B: ord[kMaxTop] u32: internal id, then d - 2*inside (steps 3-4)
-//   C: dgs[kMaxTop] u32 (degrees of the chosen vertices)
+// dynamic shared memory of the order kernel: the candidate buffer (kBytesA) and,
+// where a row is streamed, the copy of a cut
 constexpr size_t kBytesA = (size_t)kCap * 8;
-constexpr size_t kBytesB = (size_t)kMaxTop * 4;
-constexpr size_t kBytesC = (size_t)kMaxTop * 4;
-constexpr size_t kSmem = kBytesA + kBytesB + kBytesC;
-static_assert(kBytesB + kBytesC >= (size_t)kMaxTop * 8, "regions B + C hold the cut-back copy");
+constexpr size_t kSmem = kBytesA + (size_t)kMaxTop * 8;
 
 struct NcpArgs {
   const float *p = nullptr;        // [nq][n] original order
@@ -79,6 +76,17 @@ struct NcpArgs {
   double *phi = nullptr;           // [nq][top] or null
   int32_t *count = nullptr;        // [nq] or null
   unsigned long long *ncp = nullptr;  // [top] encoded profile, or null
+  // scratch of the rows of one launch
+  uint32_t *hist = nullptr;           // [rows][kBins] sampled keys per bin
+  uint32_t *edge = nullptr;           // [rows] encoded key the list starts at
+  unsigned long long *list = nullptr; // [rows][kCap] sort keys at or above it
+  uint32_t *listed = nullptr;         // [rows] their number (beyond kCap: not all are there)
+  uint32_t *positive = nullptr;       // [rows] vertices with p > 0
+  unsigned long long *part = nullptr; // [min(rows, kStreamSlots)][parts][top] a streamed row's keys by parts
+  uint32_t *kept = nullptr;           // [rows] min(top, positive)
+  uint32_t *ids = nullptr;            // [rows][top] internal ids in sweep order
+  uint32_t *first = nullptr;          // [rows][top + 1] arcs of the kept vertices before each (exclusive sums)
+  int32_t *gain = nullptr;            // [rows][top] d - 2 * inside
 };
 
 // Sort key of a vertex: FP32 bit pattern of p / max(d, 1) plus one (bit
@@ -161,8 +169,8 @@ __device__ __forceinline__ unsigned long long sort_key(uint32_t enc, uint32_t v)
 }
 
 struct Stream {
-  unsigned long long *buf;  // [kCap] candidates (region A)
-  unsigned long long *tmp;  // [kMaxTop] (regions B + C)
+  unsigned long long *buf;  // [kCap] candidates
+  unsigned long long *tmp;  // [kMaxTop]
   uint32_t *h;              // [256] digit histogram
   uint32_t *wsum;           // [kWarps]
   uint32_t *n_buf;          // candidates held
@@ -285,7 +293,7 @@ __device__ __forceinline__ float thr_key(unsigned long long thr) {
   return __uint_as_float(enc - 1u);
 }
 
-// Steps 1-2 over tiles [tlo, thi) of a row: every vertex whose sort key may
+// Tiles [tlo, thi) of a row: every vertex whose sort key may
 // still be among the T smallest is kept (the buffer holds at most T after the
 // final cut). Tiles are visited in a scrambled order: step i takes tile
 // tlo + (i * odd) mod P, P = the range rounded up to a power of two (a
@@ -350,8 +358,8 @@ __device__ void stream_row(const NcpArgs &a, const float *prow, const Stream &st
   if (*st.n_buf > T) cut_back(st, T);
 }
 
-// Merge: stream `count` keys (segments' survivors, ~0 = padding) through the
-// same buffer; at most T are held afterwards.
+// Stream `count` keys (parts' survivors, ~0 = padding) through the same buffer;
+// at most T are held afterwards.
 __device__ void stream_keys(const unsigned long long *keys, int64_t count, const Stream &st, uint32_t T) {
   for (int64_t base = 0; base < count; base += kTile) {
     const unsigned long long thr = *st.thr;
@@ -368,218 +376,493 @@ __device__ void stream_keys(const unsigned long long *keys, int64_t count, const
   if (*st.n_buf > T) cut_back(st, T);
 }
 
-struct Smem {
-  unsigned long long *cand;
-  uint32_t *hkey, *hval, *ord, *dgs;
-};
+// ---- sample -----------------------------------------------------------------
+constexpr int kBins = 4096, kBinShift = 19;     // bins of the key's FP32 bits
+constexpr int kChunk = 128;                     // row elements of a chunk (a float4 a lane)
+constexpr int kSampleEvery = 16;                // one chunk of so many, for rows of more than kSampleAll elements
+constexpr int64_t kSampleAll = 1 << 16;
+constexpr int kSampleChunks = 128;              // chunks a block samples
 
-__device__ __forceinline__ Smem carve(unsigned char *smem) {
-  Smem m;
-  m.cand = reinterpret_cast<unsigned long long *>(smem);
-  m.hkey = reinterpret_cast<uint32_t *>(smem);
-  m.hval = m.hkey + kHash;
-  m.ord = reinterpret_cast<uint32_t *>(smem + kBytesA);
-  m.dgs = reinterpret_cast<uint32_t *>(smem + kBytesA + kBytesB);
-  return m;
+__device__ __forceinline__ uint32_t chunk_hash(uint32_t c) {
+  c *= 0x9E3779B1u;
+  return c ^ (c >> 15);
 }
 
-// Steps 2-4 for row q, with the L (<= top) kept keys in cand[0, L).
-__device__ void finish_row(const NcpArgs &a, int64_t q, uint32_t L, const Smem &m);
-
-// One block per row: the whole row streamed, then steps 2-4.
-__global__ void __launch_bounds__(kThreads, 2) ncp_sweep_kernel(NcpArgs a, bool vec) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  const Smem m = carve(smem);
-  __shared__ uint32_t s_h[256], s_w32[kWarps], s_sel[2], s_n, s_m;
-  __shared__ unsigned long long s_thr;
-  const int64_t q = blockIdx.x;
-  const Stream st{m.cand, reinterpret_cast<unsigned long long *>(smem + kBytesA), s_h, s_w32, &s_n, &s_m, &s_thr, s_sel};
-  stream_begin(st);
-  const int64_t ntiles = (a.n + kTile - 1) / kTile;
-  if (vec) stream_row<true>(a, a.p + q * a.n, st, (uint32_t)a.top, 0, ntiles);
-  else stream_row<false>(a, a.p + q * a.n, st, (uint32_t)a.top, 0, ntiles);
-  finish_row(a, q, min(*st.n_buf, (uint32_t)a.top), m);
-}
-
-// `parts` blocks per row: block (q, c) keeps the top keys of segment c of row
-// q and writes them to scratch[(q * parts + c) * top ...], padded with ~0.
-__global__ void __launch_bounds__(kThreads, 2) ncp_select_kernel(NcpArgs a, bool vec, int parts,
-                                                                 unsigned long long *scratch) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  const Smem m = carve(smem);
-  __shared__ uint32_t s_h[256], s_w32[kWarps], s_sel[2], s_n, s_m;
-  __shared__ unsigned long long s_thr;
-  const int64_t q = blockIdx.x / parts;
-  const int c = (int)(blockIdx.x % parts);
-  const Stream st{m.cand, reinterpret_cast<unsigned long long *>(smem + kBytesA), s_h, s_w32, &s_n, &s_m, &s_thr, s_sel};
-  stream_begin(st);
-  const int64_t ntiles = (a.n + kTile - 1) / kTile;
-  const int64_t tlo = ntiles * c / parts, thi = ntiles * (c + 1) / parts;
-  if (vec) stream_row<true>(a, a.p + q * a.n, st, (uint32_t)a.top, tlo, thi);
-  else stream_row<false>(a, a.p + q * a.n, st, (uint32_t)a.top, tlo, thi);
-  const uint32_t held = min(*st.n_buf, (uint32_t)a.top);
-  unsigned long long *out = scratch + ((size_t)q * parts + c) * (size_t)a.top;
-  for (uint32_t i = threadIdx.x; i < (uint32_t)a.top; i += kThreads) __stcg(out + i, i < held ? m.cand[i] : ~0ull);
-}
-
-// One block per row: merge the row's `parts` segments, then steps 2-4.
-__global__ void __launch_bounds__(kThreads, 2) ncp_merge_kernel(NcpArgs a, int parts,
-                                                                const unsigned long long *scratch) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  const Smem m = carve(smem);
-  __shared__ uint32_t s_h[256], s_w32[kWarps], s_sel[2], s_n, s_m;
-  __shared__ unsigned long long s_thr;
-  const int64_t q = blockIdx.x;
-  const Stream st{m.cand, reinterpret_cast<unsigned long long *>(smem + kBytesA), s_h, s_w32, &s_n, &s_m, &s_thr, s_sel};
-  stream_begin(st);
-  stream_keys(scratch + (size_t)q * parts * (size_t)a.top, (int64_t)parts * a.top, st, (uint32_t)a.top);
-  finish_row(a, q, min(*st.n_buf, (uint32_t)a.top), m);
-}
-
-__device__ void finish_row(const NcpArgs &a, int64_t q, uint32_t L, const Smem &m) {
-  unsigned long long *cand = m.cand;
-  uint32_t *hkey = m.hkey, *hval = m.hval, *ord = m.ord, *dgs = m.dgs;
-  __shared__ unsigned long long s_w64[2][kWarps];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const uint32_t T = (uint32_t)a.top;
-  const uint32_t kmax = L;
-
-  // ---- 2. sort ----------------------------------------------------------
-  uint32_t L2 = 2;
-  while (L2 < L) L2 <<= 1;
-  for (uint32_t i = L + tid; i < L2; i += kThreads) cand[i] = ~0ull;
+// Histogram of the keys of sampled chunks: block (row, part) takes chunks
+// part * kSampleChunks and on, a warp at a time.
+template <bool VEC>
+__global__ void __launch_bounds__(kThreads) ncp_sample_kernel(NcpArgs a, int parts, int64_t chunks, int every) {
+  __shared__ uint32_t h[kBins];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t row = blockIdx.x / parts, part = blockIdx.x % parts;
+  const float *prow = a.p + row * a.n;
+  for (int i = threadIdx.x; i < kBins; i += kThreads) h[i] = 0u;
   __syncthreads();
-  for (uint32_t k = 2; k <= L2; k <<= 1) {
-    for (uint32_t j = k >> 1; j > 0; j >>= 1) {
-      for (uint32_t i = tid; i < L2; i += kThreads) {
-        const uint32_t ixj = i ^ j;
-        if (ixj > i) {
-          const unsigned long long x = cand[i], y = cand[ixj];
-          const bool up = (i & k) == 0u;
-          if ((x > y) == up) {
-            cand[i] = y;
-            cand[ixj] = x;
-          }
+  for (int64_t c = part * kSampleChunks + warp; c < chunks && c < (part + 1) * kSampleChunks; c += kWarps) {
+    const int64_t v0 = (c * every + (every > 1 ? chunk_hash((uint32_t)c) % (uint32_t)every : 0u)) * kChunk;
+    float p[4] = {0.f, 0.f, 0.f, 0.f};
+    uint32_t d[4] = {1u, 1u, 1u, 1u};
+    if (VEC) {
+      const int64_t v = v0 + 4 * lane;
+      if (v < a.n) {
+        const float4 p4 = __ldg(reinterpret_cast<const float4 *>(prow + v));
+        const uint4 d4 = __ldg(reinterpret_cast<const uint4 *>(a.deg + v));
+        p[0] = p4.x; p[1] = p4.y; p[2] = p4.z; p[3] = p4.w;
+        d[0] = d4.x; d[1] = d4.y; d[2] = d4.z; d[3] = d4.w;
+      }
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int64_t v = v0 + e * 32 + lane;
+        if (v < a.n) {
+          p[e] = __ldg(prow + v);
+          d[e] = __ldg(a.deg + v);
         }
       }
-      __syncthreads();
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const uint32_t enc = key_enc(p[e], d[e]);
+      if (enc) atomicAdd(&h[(enc - 1u) >> kBinShift], 1u);
     }
   }
-
-  // ---- 3. rank ----------------------------------------------------------
-  int32_t *orow = a.order ? a.order + q * a.top : nullptr;
-  for (uint32_t k = tid; k < kmax; k += kThreads) {
-    const uint32_t v = (uint32_t)cand[k];
-    if (orow) orow[k] = (int32_t)v;
-    const uint32_t u = a.intl ? (uint32_t)__ldg(a.intl + v) : v;
-    ord[k] = u;
-    dgs[k] = __ldg(a.rp + u + 1) - __ldg(a.rp + u);
-  }
-  __syncthreads();  // the candidate buffer is free from here on
-  for (int i = tid; i < kHash; i += kThreads) hkey[i] = kEmpty;
   __syncthreads();
-  for (uint32_t k = tid; k < kmax; k += kThreads) {
-    const uint32_t u = ord[k];
-    uint32_t s = (u * 0x9E3779B1u) >> (32 - kHashLog2);
-    for (int probe = 0; probe < kHash; ++probe, s = (s + 1) & (kHash - 1)) {
+  for (int i = threadIdx.x; i < kBins; i += kThreads)
+    if (h[i]) atomicAdd(a.hist + row * kBins + i, h[i]);
+}
+
+// Edge of each row: the highest bin edge with at least `want` sampled keys at
+// or above it (encoded key; 1 = every key, when there are fewer).
+// A row with far more keys there than the list holds (ties) is marked for the
+// stream at once: the filter would read it for nothing.
+__global__ void __launch_bounds__(kThreads) ncp_edge_kernel(NcpArgs a, uint32_t want, int every) {
+  __shared__ uint32_t w[kWarps];
+  __shared__ uint32_t s_edge;
+  const int64_t row = blockIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int kPer = kBins / kThreads;  // thread t: bins from the top, t * kPer and on
+  uint32_t c[kPer], sum = 0;
+#pragma unroll
+  for (int i = 0; i < kPer; ++i) {
+    c[i] = __ldcg(a.hist + row * kBins + (kBins - 1 - (tid * kPer + i)));
+    sum += c[i];
+  }
+  if (tid == 0) s_edge = 1u;
+  const uint32_t incl = warp_prefix_incl(sum, lane);
+  if (lane == 31) w[warp] = incl;
+  __syncthreads();
+  uint32_t above = incl - sum;
+  for (int i = 0; i < warp; ++i) above += w[i];
+#pragma unroll
+  for (int i = 0; i < kPer; ++i) {
+    if (above < want && above + c[i] >= want) {
+      s_edge = ((uint32_t)(kBins - 1 - (tid * kPer + i)) << kBinShift) + 1u;
+      if ((uint64_t)(above + c[i]) * (uint64_t)every > (uint64_t)kCap + kCap / 4) a.listed[row] = (uint32_t)kCap + 1u;
+    }
+    above += c[i];
+  }
+  __syncthreads();
+  if (tid == 0) a.edge[row] = s_edge;
+}
+
+// ---- filter -----------------------------------------------------------------
+constexpr int kFiltThreads = 256;
+constexpr int kFiltVecs = 2;     // 16-byte loads of the row in flight a thread
+constexpr int kFiltSteps = 8;    // such rounds a block
+constexpr int kFiltElems = kFiltThreads * 4 * kFiltVecs * kFiltSteps;  // row elements of a block
+constexpr int kFiltList = 3072;  // keys a block gathers; a row with more in one place is streamed instead
+
+template <bool VEC>
+__global__ void __launch_bounds__(kFiltThreads) ncp_filter_kernel(NcpArgs a, int segs) {
+  __shared__ unsigned long long s_list[kFiltList];
+  __shared__ uint32_t s_n, s_pos, s_base;
+  __shared__ bool s_skip;
+  const int64_t row = blockIdx.x / segs;
+  const int64_t lo = (blockIdx.x % segs) * (int64_t)kFiltElems;
+  const float *prow = a.p + row * a.n;
+  if (threadIdx.x == 0) {
+    s_n = 0u;
+    s_pos = 0u;
+    s_skip = __ldcg(a.listed + row) > (uint32_t)kCap;  // the row's list is not used any more
+  }
+  __syncthreads();
+  if (s_skip) return;
+  const uint32_t edge = a.edge[row];
+  // A vertex is skipped without the IEEE division when p < (K (1 - 2^-20)) * d
+  // in FP32, K = the edge's key (three roundings of at most 2^-24 each: the
+  // conversion of d and the two products, so p / d < K (1 - 2^-21) and the
+  // rounded key is below K); only while the products are normal and finite.
+  const float Kc = __fmul_rn(__uint_as_float(edge - 1u), 0x1.ffffe0p-1f);
+  const bool filt = Kc >= 1.17549435e-38f;  // FLT_MIN
+  uint32_t pos = 0;
+  for (int st = 0; st < kFiltSteps; ++st) {
+    const int64_t base = lo + (int64_t)st * kFiltThreads * 4 * kFiltVecs;
+    if (base >= a.n || *(volatile uint32_t *)&s_n > (uint32_t)kFiltList) break;
+    float p[4 * kFiltVecs];
+    uint32_t d[4 * kFiltVecs];
+    auto index = [&](int i) {
+      return VEC ? base + ((int64_t)(i >> 2) * kFiltThreads + threadIdx.x) * 4 + (i & 3)
+                 : base + (int64_t)i * kFiltThreads + threadIdx.x;
+    };
+    if (VEC) {
+#pragma unroll
+      for (int k = 0; k < kFiltVecs; ++k) {
+        const int64_t v = index(4 * k);
+        float4 p4 = make_float4(0.f, 0.f, 0.f, 0.f);
+        uint4 d4 = make_uint4(1u, 1u, 1u, 1u);
+        if (v < a.n) {  // n is a multiple of 4: the whole vector is in the row
+          p4 = __ldcs(reinterpret_cast<const float4 *>(prow + v));
+          d4 = __ldg(reinterpret_cast<const uint4 *>(a.deg + v));
+        }
+        p[4 * k] = p4.x; p[4 * k + 1] = p4.y; p[4 * k + 2] = p4.z; p[4 * k + 3] = p4.w;
+        d[4 * k] = d4.x; d[4 * k + 1] = d4.y; d[4 * k + 2] = d4.z; d[4 * k + 3] = d4.w;
+      }
+    } else {
+#pragma unroll
+      for (int i = 0; i < 4 * kFiltVecs; ++i) {
+        const int64_t v = index(i);
+        p[i] = v < a.n ? __ldcs(prow + v) : 0.f;
+        d[i] = v < a.n ? __ldg(a.deg + v) : 1u;
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 4 * kFiltVecs; ++i) {
+      if (!(p[i] > 0.f)) continue;
+      ++pos;
+      if (filt) {
+        const float lim = __fmul_rn(Kc, __uint2float_rn(d[i] > 0u ? d[i] : 1u));
+        if (lim <= 3.40282347e+38f && p[i] < lim) continue;
+      }
+      const uint32_t enc = key_enc(p[i], d[i]);
+      if (enc < edge) continue;
+      const unsigned long long key = sort_key(enc, (uint32_t)index(i));
+      const uint32_t at = atomicAdd(&s_n, 1u);
+      if (at < (uint32_t)kFiltList) s_list[at] = key;
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) pos += __shfl_xor_sync(0xFFFFFFFFu, pos, o);
+  if ((threadIdx.x & 31) == 0 && pos) atomicAdd(&s_pos, pos);
+  __syncthreads();
+  if (s_n > (uint32_t)kFiltList) {
+    if (threadIdx.x == 0) atomicAdd(a.listed + row, (uint32_t)kCap + 1u);
+    return;
+  }
+  const uint32_t n = s_n;
+  if (threadIdx.x == 0) {
+    if (s_pos) atomicAdd(a.positive + row, s_pos);
+    s_base = n ? atomicAdd(a.listed + row, n) : 0u;
+  }
+  __syncthreads();
+  for (uint32_t i = threadIdx.x; i < n; i += kFiltThreads)
+    if (s_base + i < (uint32_t)kCap) a.list[row * kCap + s_base + i] = s_list[i];
+}
+
+// ---- order ------------------------------------------------------------------
+// Place of the i-th key of a sorted buffer: sixteen consecutive keys lie in
+// sixteen different banks' places, and so do the same ones of sixteen groups.
+__device__ __forceinline__ uint32_t sort_place(uint32_t i) { return i ^ ((i >> 4) & 15u); }
+
+// `kN` halving steps of a bitonic merge of runs of k keys, distances j, j / 2, ...:
+// a thread takes the 2^kN keys that meet in them, so that shared memory and the
+// barrier are passed once.
+template <int kN>
+__device__ __forceinline__ void merge_steps(unsigned long long *cand, uint32_t L2, uint32_t k, uint32_t j) {
+  constexpr int kM = 1 << kN;
+  const uint32_t step = j >> (kN - 1);
+  for (uint32_t t = threadIdx.x; t < (L2 >> kN); t += kThreads) {
+    const uint32_t base = ((t & ~(step - 1u)) << kN) | (t & (step - 1u));
+    const bool up = (base & k) == 0u;  // (k is above every distance: the same for all of them)
+    unsigned long long x[kM];
+#pragma unroll
+    for (int m = 0; m < kM; ++m) x[m] = cand[sort_place(base + (uint32_t)m * step)];
+#pragma unroll
+    for (int h = kM / 2; h > 0; h >>= 1) {
+#pragma unroll
+      for (int m = 0; m < kM; ++m) {
+        if (m & h) continue;
+        const unsigned long long a = x[m], b = x[m | h];
+        const bool swap = (a > b) == up;
+        x[m] = swap ? b : a;
+        x[m | h] = swap ? a : b;
+      }
+    }
+#pragma unroll
+    for (int m = 0; m < kM; ++m) cand[sort_place(base + (uint32_t)m * step)] = x[m];
+  }
+  __syncthreads();
+}
+
+// Sorts the keys in cand[0, L) ascending (padded to a power of two of at least
+// 16, at most kCap; block-wide): the i-th is then at cand[sort_place(i)].
+__device__ void sort_keys(unsigned long long *cand, uint32_t L) {
+  uint32_t L2 = 16;
+  while (L2 < L) L2 <<= 1;
+  for (uint32_t i = L + threadIdx.x; i < L2; i += kThreads) cand[i] = ~0ull;
+  __syncthreads();
+  for (uint32_t k = 2; k <= L2; k <<= 1) {
+    uint32_t j = k >> 1;
+    for (; j >= 8; j >>= 4) merge_steps<4>(cand, L2, k, j);
+    if (j == 4) merge_steps<3>(cand, L2, k, j);
+    if (j == 2) merge_steps<2>(cand, L2, k, j);
+    if (j == 1) merge_steps<1>(cand, L2, k, j);
+  }
+}
+
+// The first L sorted keys of a row: put(k, id, degree) in sweep order, then
+// sum(k, arcs before k) for k in [0, L] (a graph has fewer than 2^32 arcs).
+// Overwrites the keys; block-wide.
+template <class Put, class Sum>
+__device__ __forceinline__ void write_order(const NcpArgs &a, int64_t row, unsigned long long *cand, uint32_t L,
+                                            uint32_t *s_w32, Put put, Sum sum_at) {
+  int32_t *orow = a.order ? a.order + row * a.top : nullptr;
+  const uint32_t per = (L + kThreads - 1) / kThreads;
+  const uint32_t k0 = min(L, threadIdx.x * per), k1 = min(L, k0 + per);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint32_t sum = 0;
+  for (uint32_t k = k0; k < k1; ++k) {
+    const uint32_t v = (uint32_t)cand[sort_place(k)], u = a.intl ? (uint32_t)__ldg(a.intl + v) : v;
+    const uint32_t arc = __ldg(a.rp + u), deg = __ldg(a.rp + u + 1) - arc;
+    if (orow) orow[k] = (int32_t)v;
+    put(k, u, arc, deg);
+    sum += deg;
+    cand[sort_place(k)] = deg;  // (its key has been read)
+  }
+  const uint32_t incl = warp_prefix_incl(sum, lane);
+  if (lane == 31) s_w32[warp] = incl;
+  __syncthreads();
+  uint32_t before = incl - sum;
+  for (int w = 0; w < warp; ++w) before += s_w32[w];
+  for (uint32_t k = k0; k < k1; ++k) {
+    sum_at(k, before);
+    before += (uint32_t)cand[sort_place(k)];
+  }
+  if (threadIdx.x == kThreads - 1) sum_at(L, before);  // its share is the last one, empty or not
+}
+
+// A row whose list cannot be used is streamed, the first kStreamSlots rows of a
+// launch in parts, by up to kStreamParts blocks each.
+constexpr int kStreamParts = 16;
+constexpr int64_t kStreamSlots = 128;
+
+__device__ __forceinline__ bool list_usable(const NcpArgs &a, int64_t row) {
+  return a.listed[row] <= (uint32_t)kCap && a.listed[row] >= min((uint32_t)a.top, a.positive[row]);
+}
+
+struct RowStream {
+  uint32_t h[256], w32[kWarps], sel[2], n, m;
+  unsigned long long thr;
+  __device__ Stream on(unsigned char *smem) {
+    return Stream{reinterpret_cast<unsigned long long *>(smem), reinterpret_cast<unsigned long long *>(smem + kBytesA),
+                  h, w32, &n, &m, &thr, sel};
+  }
+};
+
+__device__ __forceinline__ void stream_part(const NcpArgs &a, int64_t row, bool vec, const Stream &st, int part,
+                                            int parts) {
+  const int64_t ntiles = (a.n + kTile - 1) / kTile, lo = ntiles * part / parts, hi = ntiles * (part + 1) / parts;
+  if (vec) stream_row<true>(a, a.p + row * a.n, st, (uint32_t)a.top, lo, hi);
+  else stream_row<false>(a, a.p + row * a.n, st, (uint32_t)a.top, lo, hi);
+}
+
+__global__ void __launch_bounds__(kThreads, 2) ncp_stream_kernel(NcpArgs a, bool vec, int parts) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ RowStream rs;
+  const int64_t row = blockIdx.x / parts;
+  const int part = (int)(blockIdx.x % parts);
+  if (list_usable(a, row)) return;
+  const Stream st = rs.on(smem);
+  stream_begin(st);
+  stream_part(a, row, vec, st, part, parts);
+  const uint32_t held = min(*st.n_buf, (uint32_t)a.top);
+  unsigned long long *out = a.part + ((size_t)row * parts + part) * (size_t)a.top;
+  for (uint32_t i = threadIdx.x; i < (uint32_t)a.top; i += kThreads) __stcg(out + i, i < held ? st.buf[i] : ~0ull);
+}
+
+__global__ void __launch_bounds__(kThreads, 2) ncp_order_kernel(NcpArgs a, bool vec, int parts) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  unsigned long long *cand = reinterpret_cast<unsigned long long *>(smem);
+  __shared__ RowStream rs;
+  uint32_t *s_w32 = rs.w32;
+  const int64_t row = blockIdx.x;
+  const uint32_t T = (uint32_t)a.top;
+  uint32_t L;
+  if (list_usable(a, row)) {
+    L = a.listed[row];
+    for (uint32_t i = threadIdx.x; i < L; i += kThreads) cand[i] = __ldcg(a.list + row * kCap + i);
+    __syncthreads();
+  } else {
+    const Stream st = rs.on(smem);
+    stream_begin(st);
+    if (row < kStreamSlots)
+      stream_keys(a.part + (size_t)row * parts * (size_t)a.top, (int64_t)parts * a.top, st, T);
+    else
+      stream_part(a, row, vec, st, 0, 1);
+    L = min(*st.n_buf, T);
+  }
+  sort_keys(cand, L);
+  L = min(L, T);
+  if (threadIdx.x == 0) a.kept[row] = L;
+  write_order(
+      a, row, cand, L, s_w32,
+      [&](uint32_t k, uint32_t u, uint32_t, uint32_t deg) {
+        a.ids[row * a.top + k] = u;
+        a.gain[row * a.top + k] = (int32_t)deg;
+      },
+      [&](uint32_t k, uint32_t before) { a.first[row * ((int64_t)a.top + 1) + k] = before; });
+}
+
+// ---- inside -------------------------------------------------------------------
+// The arcs of a row's kept vertices are one run, cut into pieces of kInsideArcs
+// so that a hub's arcs are spread over blocks: block (row, part) takes pieces
+// part, part + parts, ..., and leaves at once where there are fewer. An arc's
+// owner is found by halving in the sums of the degrees, once for a thread's
+// four arcs. Few of the neighbours are in the set, so two bits of a bitmap (32
+// a member) are asked before the hash, whose probes for an absent vertex run to
+// the next empty slot and keep the warp; a neighbour ranked before its vertex
+// takes two from the vertex's gain.
+constexpr int kInsideThreads = 1024;
+constexpr uint32_t kInsideArcs = 1u << 15;
+constexpr int kInsideParts = 16;
+constexpr int kBitsLog2 = 17;
+// hash keys and ranks, bitmap, first arc of each member in the run and in the graph
+constexpr size_t kInsideSmem =
+    (size_t)kHash * 6 + ((size_t)1 << kBitsLog2) / 8 + 2 * (size_t)kMaxTop * 4;
+static_assert(kMaxTop <= 1 << 16, "ranks of 16 bits");
+
+__device__ __forceinline__ uint32_t bit_a(uint32_t x, int shift) { return x >> shift; }
+__device__ __forceinline__ uint32_t bit_b(uint32_t u, int shift) { return (u * 0x85EBCA6Bu) >> shift; }
+
+// The kept vertices of a row in shared memory; the hash has at least twice as
+// many slots as members, the bitmap sixteen bits a slot.
+struct Members {
+  uint32_t *hkey, *bits, *first, *arc;
+  uint16_t *hval;
+  uint32_t L, hmask;
+  int hshift, bshift;
+
+  __device__ Members(unsigned char *smem, uint32_t count) {
+    hkey = reinterpret_cast<uint32_t *>(smem);
+    bits = hkey + kHash;
+    first = bits + (1 << kBitsLog2) / 32;
+    arc = first + kMaxTop;
+    hval = reinterpret_cast<uint16_t *>(arc + kMaxTop);
+    L = count;
+    int log2 = 8;
+    while ((1u << log2) < 2u * L) ++log2;
+    hmask = (1u << log2) - 1u;
+    hshift = 32 - log2;
+    bshift = hshift - (kBitsLog2 - kHashLog2);
+  }
+  __device__ void clear(int threads) {
+    for (uint32_t i = threadIdx.x; i <= hmask; i += threads) hkey[i] = kEmpty;
+    for (uint32_t i = threadIdx.x; i < (1u << (32 - bshift)) / 32u; i += threads) bits[i] = 0u;
+    for (uint32_t i = L + threadIdx.x; i < (uint32_t)kMaxTop; i += threads) first[i] = 0xFFFFFFFFu;  // beyond every arc
+  }
+  __device__ void insert(uint32_t i, uint32_t u) {
+    const uint32_t x = u * 0x9E3779B1u;
+    atomicOr(&bits[bit_a(x, bshift) >> 5], 1u << (bit_a(x, bshift) & 31));
+    atomicOr(&bits[bit_b(u, bshift) >> 5], 1u << (bit_b(u, bshift) & 31));
+    uint32_t s = x >> hshift;
+    for (uint32_t probe = 0; probe <= hmask; ++probe, s = (s + 1) & hmask) {
       if (atomicCAS(&hkey[s], kEmpty, u) == kEmpty) {
-        hval[s] = k;
+        hval[s] = (uint16_t)i;
         break;
       }
     }
   }
-  __syncthreads();
-  // neighbours ranked before k. The sweep set mixes many light vertices with a
-  // few hubs (tens of thousands of arcs), so the count is split three ways:
-  // a light vertex (<= 32 arcs) is counted by one lane, so that 32 vertices'
-  // load chains are in flight per warp; a medium one by its warp; a hub
-  // (more than kBlockArcs arcs) by the whole block, after the rest. Every
-  // thread keeps 4 arc loads in flight before it probes the hash.
-  constexpr uint32_t kBlockArcs = 4096;
-  constexpr int kMaxHubs = 64;
-  __shared__ uint32_t s_hub[kMaxHubs], s_nhub, s_red[kWarps];
-  auto ranked_before = [&](uint32_t w, uint32_t k) -> uint32_t {
-    uint32_t sl = (w * 0x9E3779B1u) >> (32 - kHashLog2);
-    for (int probe = 0; probe < kHash; ++probe, sl = (sl + 1) & (kHash - 1)) {
-      const uint32_t hk = hkey[sl];
-      if (hk == w) return hval[sl] < k ? 1u : 0u;
-      if (hk == kEmpty) return 0u;
-    }
-    return 0u;
-  };
-  // arcs [b, e1) with stride `step`, 4 loads in flight per thread
-  auto count_arcs = [&](uint32_t b, uint32_t e1, uint32_t step, uint32_t k) -> uint32_t {
-    uint32_t inside = 0;
-    for (uint32_t e = b; e < e1; e += 4 * step) {
-      uint32_t w4[4];
+  // Arcs [begin, end) of the members' run, by a block of kT threads: four
+  // consecutive ones a lane. A hub's arcs fill warps, whose lanes then add
+  // their counts first (32 atomics on one word take their turns).
+  template <int kT>
+  __device__ void count(const uint32_t *adj, uint32_t begin, uint32_t end, int32_t *gain) const {
+    constexpr int kU = 4;
+    const int lane = threadIdx.x & 31;
+    // (64 bits: begin + kT * kU may lie past 2^32)
+    for (uint64_t base = begin + (uint64_t)(threadIdx.x & ~31u) * kU; base < end; base += kT * kU) {
+      const uint64_t t0 = base + (uint64_t)lane * kU;
+      uint32_t lo = 0;  // last member whose arcs start at or before t0 (those without arcs share a start)
+      const uint32_t tc = (uint32_t)min(t0, (uint64_t)end - 1u);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) w4[j] = e + j * step < e1 ? __ldg(a.adj + e + j * step) : kEmpty;
+      for (uint32_t half = kMaxTop / 2; half; half >>= 1)
+        if (first[lo + half] <= tc) lo += half;
+      uint32_t w[kU], own[kU];
 #pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (w4[j] != kEmpty) inside += ranked_before(w4[j], k);
-    }
-    return inside;
-  };
-  if (tid == 0) s_nhub = 0;
-  __syncthreads();
-  for (uint32_t k0 = warp * 32; k0 < kmax; k0 += kWarps * 32) {
-    const uint32_t k = k0 + lane;
-    uint32_t e0 = 0, e1 = 0;
-    if (k < kmax) {
-      const uint32_t u = ord[k];
-      e0 = __ldg(a.rp + u);
-      e1 = __ldg(a.rp + u + 1);
-    }
-    const bool light = k < kmax && e1 - e0 <= 32u;
-    if (light) ord[k] = (uint32_t)((int32_t)dgs[k] - 2 * (int32_t)count_arcs(e0, e1, 1u, k));
-    unsigned heavy = __ballot_sync(0xFFFFFFFFu, k < kmax && !light);
-    while (heavy) {
-      const int j = __ffs(heavy) - 1;
-      heavy &= heavy - 1;
-      const uint32_t kh = k0 + j;
-      const uint32_t h0 = __shfl_sync(0xFFFFFFFFu, e0, j), h1 = __shfl_sync(0xFFFFFFFFu, e1, j);
-      if (h1 - h0 > kBlockArcs) {
-        uint32_t slot = 0;
-        if (lane == 0) slot = atomicAdd(&s_nhub, 1u);
-        slot = __shfl_sync(0xFFFFFFFFu, slot, 0);
-        if (slot < (uint32_t)kMaxHubs) {
-          if (lane == 0) s_hub[slot] = kh;  // counted by the block below
-          continue;
+      for (int i = 0; i < kU; ++i) {
+        const uint64_t t = t0 + (uint64_t)i;
+        w[i] = kEmpty;
+        if (t < end) {
+          while (lo + 1u < L && first[lo + 1u] <= (uint32_t)t) ++lo;
+          w[i] = __ldg(adj + arc[lo] + ((uint32_t)t - first[lo]));
+        }
+        own[i] = lo;
+      }
+      uint32_t of = own[0];
+      int32_t inside = 0;
+#pragma unroll
+      for (int i = 0; i < kU; ++i) {
+        if (own[i] != of) {
+          if (inside) atomicAdd(gain + of, -2 * inside);
+          of = own[i];
+          inside = 0;
+        }
+        const uint32_t x = w[i] * 0x9E3779B1u, ba = bit_a(x, bshift), bb = bit_b(w[i], bshift);
+        const bool may = ((bits[ba >> 5] >> (ba & 31)) & (bits[bb >> 5] >> (bb & 31)) & 1u) != 0u;
+        if (!may || w[i] == kEmpty) continue;
+        uint32_t s = x >> hshift;
+        for (uint32_t probe = 0; probe <= hmask; ++probe, s = (s + 1) & hmask) {
+          const uint32_t hk = hkey[s];
+          if (hk == w[i] && hval[s] < own[i]) ++inside;
+          if (hk == w[i] || hk == kEmpty) break;
         }
       }
-      uint32_t inside = count_arcs(h0 + lane, h1, 32u, kh);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) inside += __shfl_xor_sync(0xFFFFFFFFu, inside, o);
-      if (lane == j) ord[kh] = (uint32_t)((int32_t)dgs[kh] - 2 * (int32_t)inside);
+      __syncwarp();
+      if (__all_sync(0xFFFFFFFFu, of == __shfl_sync(0xFFFFFFFFu, of, 0))) {
+        inside = __reduce_add_sync(0xFFFFFFFFu, inside);
+        if (lane == 0 && inside) atomicAdd(gain + of, -2 * inside);
+      } else if (inside) {
+        atomicAdd(gain + of, -2 * inside);
+      }
     }
+  }
+};
+
+__global__ void __launch_bounds__(kInsideThreads, 2) ncp_inside_kernel(NcpArgs a, int parts) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int64_t row = blockIdx.x / parts;
+  const uint32_t L = a.kept[row], *first = a.first + row * ((int64_t)a.top + 1), tot = first[L];
+  uint64_t at = (uint64_t)(blockIdx.x % parts) * kInsideArcs;
+  if (at >= tot) return;
+  Members m(smem, L);
+  m.clear(kInsideThreads);
+  __syncthreads();
+  for (uint32_t i = threadIdx.x; i < L; i += kInsideThreads) {
+    const uint32_t u = a.ids[row * a.top + i];
+    m.first[i] = first[i];
+    m.arc[i] = __ldg(a.rp + u);
+    m.insert(i, u);
   }
   __syncthreads();
-  const uint32_t nhub = min(s_nhub, (uint32_t)kMaxHubs);
-  for (uint32_t i = 0; i < nhub; ++i) {
-    const uint32_t kh = s_hub[i];
-    // ord[kh] still holds the hub's internal id: every thread reads it before the write below
-    const uint32_t u = ord[kh];
-    const uint32_t h0 = __ldg(a.rp + u), h1 = __ldg(a.rp + u + 1);
-    uint32_t inside = count_arcs(h0 + tid, h1, kThreads, kh);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) inside += __shfl_xor_sync(0xFFFFFFFFu, inside, o);
-    if (lane == 0) s_red[warp] = inside;
-    __syncthreads();
-    if (tid == 0) {
-      uint32_t tot = 0;
-      for (int w = 0; w < kWarps; ++w) tot += s_red[w];
-      ord[kh] = (uint32_t)((int32_t)dgs[kh] - 2 * (int32_t)tot);
-    }
-    __syncthreads();
-  }
+  for (; at < tot; at += (uint64_t)parts * kInsideArcs)
+    m.count<kInsideThreads>(a.adj, (uint32_t)at, (uint32_t)min(at + kInsideArcs, (uint64_t)tot), a.gain + row * a.top);
+}
 
-  // ---- 4. scan ----------------------------------------------------------
+// ---- scan ---------------------------------------------------------------------
+// kmax vertices kept; degree(k), gain(k) = degree(k) - 2 * inside(k).
+template <class Degree>
+__device__ __forceinline__ void scan_row(const NcpArgs &a, int64_t row, uint32_t kmax, const int32_t *gain,
+                                         Degree degree) {
+  __shared__ unsigned long long s_w64[2][kWarps];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t T = (uint32_t)a.top;
+  int32_t *orow = a.order ? a.order + row * a.top : nullptr;
+  double *prow_phi = a.phi ? a.phi + row * a.top : nullptr;
   const uint32_t per = (kmax + kThreads - 1) / kThreads;
   const uint32_t k0 = min(kmax, (uint32_t)tid * per), k1 = min(kmax, k0 + per);
   long long cut_t = 0, vol_t = 0;
   for (uint32_t k = k0; k < k1; ++k) {
-    cut_t += (int32_t)ord[k];
-    vol_t += dgs[k];
+    cut_t += gain[k];
+    vol_t += degree(k);
   }
   const long long cut_i = warp_prefix_incl(cut_t, lane), vol_i = warp_prefix_incl(vol_t, lane);
   if (lane == 31) {
@@ -593,10 +876,9 @@ __device__ void finish_row(const NcpArgs &a, int64_t q, uint32_t L, const Smem &
     vol += (long long)s_w64[1][w];
   }
   const long long vol_all = (long long)a.m;
-  double *prow_phi = a.phi ? a.phi + q * a.top : nullptr;
   for (uint32_t k = k0; k < k1; ++k) {
-    cut += (int32_t)ord[k];
-    vol += dgs[k];
+    cut += gain[k];
+    vol += degree(k);
     const long long rest = vol_all - vol;
     const long long den = vol < rest ? vol : rest;
     const double phi = den > 0 ? (double)cut / (double)den : 1.0;
@@ -607,7 +889,67 @@ __device__ void finish_row(const NcpArgs &a, int64_t q, uint32_t L, const Smem &
     if (orow) orow[k] = -1;
     if (prow_phi) prow_phi[k] = __longlong_as_double(0x7FF8000000000000ll);  // NaN: no such prefix
   }
-  if (tid == 0 && a.count) a.count[q] = (int32_t)kmax;
+  if (tid == 0 && a.count) a.count[row] = (int32_t)kmax;
+}
+
+__global__ void __launch_bounds__(kThreads) ncp_scan_kernel(NcpArgs a) {
+  const int64_t row = blockIdx.x;
+  const uint32_t *first = a.first + row * ((int64_t)a.top + 1);
+  scan_row(a, row, a.kept[row], a.gain + row * a.top, [&](uint32_t k) { return first[k + 1] - first[k]; });
+}
+
+// ---- rows of few vertices -------------------------------------------------------
+// Everything for a row in one block and its shared memory, for rows of at most
+// kSmallRow vertices: what the kernels above take there is mostly their launches.
+// 9,000 vertices, 1 row, top 300: 44 us here and 72 through them; at the line the
+// two meet (105 rows, top 4,096: 263 us here with 16,000 vertices, 255 through
+// them with 17,000).
+constexpr int64_t kSmallRow = 1 << 14;
+constexpr size_t kSmallSmem = kInsideSmem + (size_t)kMaxTop * 4;  // and the gains
+static_assert(kSmem <= kSmallSmem, "the row is streamed in the same memory");
+
+__global__ void __launch_bounds__(kThreads) ncp_small_kernel(NcpArgs a, bool vec) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  unsigned long long *cand = reinterpret_cast<unsigned long long *>(smem);
+  __shared__ RowStream rs;
+  __shared__ uint32_t s_tot;
+  const int64_t row = blockIdx.x;
+  const Stream st = rs.on(smem);
+  stream_begin(st);
+  stream_part(a, row, vec, st, 0, 1);
+  const uint32_t L = min(*st.n_buf, (uint32_t)a.top);
+  sort_keys(cand, L);
+  // the sorted keys take the first kMaxTop * 8 bytes, hash keys later; the
+  // vertices themselves wait in registers
+  Members m(smem, L);
+  int32_t *gain = reinterpret_cast<int32_t *>(smem + kInsideSmem);
+  constexpr int kPer = kMaxTop / kThreads;
+  uint32_t id[kPer];
+  const uint32_t per = (L + kThreads - 1) / kThreads, k0 = min(L, threadIdx.x * per);
+  write_order(
+      a, row, cand, L, rs.w32,
+      [&](uint32_t k, uint32_t u, uint32_t arc, uint32_t deg) {
+#pragma unroll
+        for (int i = 0; i < kPer; ++i)
+          if (k - k0 == (uint32_t)i) id[i] = u;
+        m.arc[k] = arc;
+        gain[k] = (int32_t)deg;
+      },
+      [&](uint32_t k, uint32_t before) {
+        if (k < L) m.first[k] = before;
+        else s_tot = before;
+      });
+  __syncthreads();
+  m.clear(kThreads);
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < kPer; ++i)
+    if ((uint32_t)i < per && k0 + (uint32_t)i < L) m.insert(k0 + (uint32_t)i, id[i]);
+  __syncthreads();
+  const uint32_t tot = s_tot;
+  m.count<kThreads>(a.adj, 0u, tot, gain);
+  __syncthreads();
+  scan_row(a, row, L, gain, [&](uint32_t k) { return (k + 1u < L ? m.first[k + 1u] : tot) - m.first[k]; });
 }
 
 // profile: accumulate ? encode the caller's values : start from +inf (encoded)
@@ -665,11 +1007,15 @@ extern "C" fg_status fg_ncp_sweep(fg_graph *g, const float *p, int32_t nq, int32
       static std::once_flag attr_once;
       static cudaError_t attr_err = cudaSuccess;
       std::call_once(attr_once, [] {
-        attr_err = cudaFuncSetAttribute(ncp_sweep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+        attr_err = cudaFuncSetAttribute(ncp_order_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
         if (attr_err == cudaSuccess)
-          attr_err = cudaFuncSetAttribute(ncp_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+          attr_err = cudaFuncSetAttribute(ncp_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
         if (attr_err == cudaSuccess)
-          attr_err = cudaFuncSetAttribute(ncp_merge_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+          attr_err = cudaFuncSetAttribute(ncp_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)kSmallSmem);
+        if (attr_err == cudaSuccess)
+          attr_err = cudaFuncSetAttribute(ncp_inside_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)kInsideSmem);
       });
       CUDA_TRY(attr_err);
       DevBuf d;
@@ -704,30 +1050,82 @@ extern "C" fg_status fg_ncp_sweep(fg_graph *g, const float *p, int32_t nq, int32
     CUDA_TRY(cudaGetLastError());
   }
   const bool vec = (n % 4 == 0) && aligned(p, 16);
-  // Rows are split into `parts` segments when there are too few rows to give
-  // every SM two blocks: each segment's block keeps its top keys, and one
-  // block per row merges them (the kept set does not depend on the split).
-  int sms = 0;
-  CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const int64_t ntiles = (n + kTile - 1) / kTile;
-  int64_t parts = (4ll * sms + nq - 1) / nq;
-  parts = std::min<int64_t>(std::min<int64_t>(parts, 16), ntiles / 4);
-  if (parts <= 1) {
-    ncp_sweep_kernel<<<nq, kThreads, kSmem, stream>>>(a, vec);
-    CUDA_TRY(cudaGetLastError());
-  } else {
-    unsigned long long *scratch = nullptr;
-    const size_t bytes = (size_t)nq * (size_t)parts * (size_t)top * sizeof(unsigned long long);
-    CUDA_TRY(cudaMallocAsync(reinterpret_cast<void **>(&scratch), bytes, stream));
-    ncp_select_kernel<<<(unsigned)(nq * parts), kThreads, kSmem, stream>>>(a, vec, (int)parts, scratch);
-    cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) {
-      ncp_merge_kernel<<<nq, kThreads, kSmem, stream>>>(a, (int)parts, scratch);
-      e = cudaGetLastError();
-    }
-    cudaFreeAsync(scratch, stream);
-    CUDA_TRY(e);
+  // Rows go through in launches of at most kRowsPerLaunch, which bounds the
+  // scratch (about 80 KB + 12 * top bytes a row, from the stream-ordered
+  // allocator).
+  constexpr int64_t kRowsPerLaunch = 1024;
+  const bool small = n <= kSmallRow;
+  auto up = [](size_t b) { return (b + 255) / 256 * 256; };
+  int64_t rows_max = std::min<int64_t>(nq, kRowsPerLaunch);
+  size_t b_hist = 0, b_small = 0, b_list = 0, b_top = 0, b_part = 0;
+  int stream_parts = 0;
+  unsigned char *scratch = nullptr;
+  for (; !small; rows_max = (rows_max + 1) / 2) {  // fewer rows a launch where memory is short
+    b_hist = up((size_t)rows_max * kBins * 4);
+    b_small = up((size_t)rows_max * 4);
+    b_list = up((size_t)rows_max * kCap * 8);
+    b_top = up((size_t)rows_max * ((size_t)top + 1) * 4);
+    stream_parts = (int)std::max<int64_t>(1, std::min<int64_t>(kStreamParts, 304 / rows_max));  // two blocks an SM
+    b_part = up((size_t)std::min(rows_max, kStreamSlots) * (size_t)stream_parts * (size_t)top * 8);
+    const cudaError_t e0 = cudaMallocAsync(reinterpret_cast<void **>(&scratch),
+                                           b_hist + 4 * b_small + b_list + 3 * b_top + b_part, stream);
+    if (e0 == cudaSuccess) break;
+    if (e0 != cudaErrorMemoryAllocation || rows_max == 1) CUDA_TRY(e0);
+    (void)cudaGetLastError();
   }
+  unsigned char *at = scratch;
+  auto take = [&at](size_t b) {
+    unsigned char *r = at;
+    at += b;
+    return r;
+  };
+  // (listed, positive and hist start at zero: one memset)
+  a.listed = reinterpret_cast<uint32_t *>(take(b_small));
+  a.positive = reinterpret_cast<uint32_t *>(take(b_small));
+  a.hist = reinterpret_cast<uint32_t *>(take(b_hist));
+  a.edge = reinterpret_cast<uint32_t *>(take(b_small));
+  a.kept = reinterpret_cast<uint32_t *>(take(b_small));
+  a.list = reinterpret_cast<unsigned long long *>(take(b_list));
+  a.ids = reinterpret_cast<uint32_t *>(take(b_top));
+  a.gain = reinterpret_cast<int32_t *>(take(b_top));
+  a.first = reinterpret_cast<uint32_t *>(take(b_top));
+  a.part = reinterpret_cast<unsigned long long *>(take(b_part));
+  const int every = n > kSampleAll ? kSampleEvery : 1;
+  const int64_t chunks = (n / every + kChunk - 1) / kChunk;  // (a sampled row's last chunks may lie past its end)
+  const int sparts = (int)((chunks + kSampleChunks - 1) / kSampleChunks);
+  // keys wanted above the edge among the sampled ones: with one in sixteen, the
+  // share of `top` and six standard deviations of it, and a tenth of room
+  const double share = (double)top / every;
+  const uint32_t want = every == 1 ? (uint32_t)top : (uint32_t)(1.1 * share + 6.0 * std::sqrt(share) + 8.0);
+  const int segs = (int)((n + kFiltElems - 1) / kFiltElems);
+  cudaError_t e = cudaSuccess;
+  for (int64_t r0 = 0; r0 < nq && e == cudaSuccess; r0 += rows_max) {
+    const unsigned rows = (unsigned)std::min<int64_t>(rows_max, nq - r0);
+    NcpArgs b = a;
+    b.p = a.p + r0 * n;
+    if (a.order) b.order = a.order + r0 * top;
+    if (a.phi) b.phi = a.phi + r0 * top;
+    if (a.count) b.count = a.count + r0;
+    if (small) {
+      ncp_small_kernel<<<rows, kThreads, kSmallSmem, stream>>>(b, vec);
+      e = cudaGetLastError();
+      continue;
+    }
+    e = cudaMemsetAsync(scratch, 0, 2 * b_small + b_hist, stream);
+    if (vec) ncp_sample_kernel<true><<<rows * sparts, kThreads, 0, stream>>>(b, sparts, chunks, every);
+    else ncp_sample_kernel<false><<<rows * sparts, kThreads, 0, stream>>>(b, sparts, chunks, every);
+    ncp_edge_kernel<<<rows, kThreads, 0, stream>>>(b, want, every);
+    if (vec) ncp_filter_kernel<true><<<rows * segs, kFiltThreads, 0, stream>>>(b, segs);
+    else ncp_filter_kernel<false><<<rows * segs, kFiltThreads, 0, stream>>>(b, segs);
+    const unsigned streamed = (unsigned)std::min<int64_t>(rows, kStreamSlots);
+    ncp_stream_kernel<<<streamed * stream_parts, kThreads, kSmem, stream>>>(b, vec, stream_parts);
+    ncp_order_kernel<<<rows, kThreads, kSmem, stream>>>(b, vec, stream_parts);
+    ncp_inside_kernel<<<rows * kInsideParts, kInsideThreads, kInsideSmem, stream>>>(b, kInsideParts);
+    ncp_scan_kernel<<<rows, kThreads, 0, stream>>>(b);
+    if (e == cudaSuccess) e = cudaGetLastError();
+  }
+  if (scratch) cudaFreeAsync(scratch, stream);
+  CUDA_TRY(e);
   if (a.ncp) {
     ncp_profile_end<<<(top + 255) / 256, 256, 0, stream>>>(a.ncp, top);
     CUDA_TRY(cudaGetLastError());
