@@ -13,9 +13,11 @@
 //                       per row; the padded tile keeps both phases free of bank
 //                       conflicts), persistent blocks that load the next tile
 //                       while writing the current one; 8 * K * n bytes;
-//   query               one warp per pair reads the two K-entry labels with
-//                       16-byte loads (K a multiple of 4) and reduces the
-//                       minimum with shuffles; 8 * K + 16 bytes per pair.
+//   query               few pairs: one warp per pair reads the two K-entry
+//                       labels with 16-byte loads (K a multiple of 4) and
+//                       reduces the minimum with shuffles; 8 * K + 16 bytes per
+//                       pair. Many: the labels are taken in slices of columns
+//                       that stay in L2 while all pairs use them.
 #include <algorithm>
 #include <cstdint>
 
@@ -115,6 +117,110 @@ __global__ void __launch_bounds__(kQThreads) ll_query_kernel(const uint32_t *__r
   }
 }
 
+// Many pairs: a warp keeps up to kMine of them with their minima in shared memory
+// and takes the labels in slices of kLanes * kC columns, kLanes lanes a pair, kC
+// columns a lane, 32 words of a lane in flight. All blocks are resident and have
+// the same number of pairs, so they stay on the same few slices, which L2 holds:
+// a label is read from HBM once and not once a pair, and a pair with few columns
+// does not take a whole warp. Sums are taken in 32 bits while one of a pair's
+// stays below 2^32 - 1 (it is then the least of all).
+//   n = 2^18, K = 1,024, Q = 2^20  1.15 ms (7.4 TB/s) -> 0.75  (8.6 GB of labels, 1.07 GB once)
+//   n = 2^15 (labels in L2)        0.67 -> 0.45
+//   n = 2^18, K = 1,023            1.61 -> 1.12  (no 16-byte loads)
+//   n = 2^18, K = 64 / 16          170 us -> 35 / 158 -> 17
+// Slices of 128 columns (64 where K ends there): with 64 and 256 the first line is
+// 0.81 and 0.92. Below kSliceMinPairs a warp per pair is the faster one:
+// Q = 4,000 of the first line 6.3 us and 25; 10,000 pairs of 9 columns 4.7 and 6.5;
+// 32,768 pairs 45.2 and 42.8 (K = 1,024), 65.7 and 47.6 (1,023).
+constexpr int kMine = 256;
+constexpr int64_t kSliceMinPairs = 1 << 15;
+constexpr int64_t kSliceBlocks = 152 * 4;
+
+template <bool VEC, int kLanes, int kC>
+__global__ void __launch_bounds__(kQThreads, 4) ll_slice_kernel(const uint32_t *__restrict__ labels, int64_t n, int32_t K,
+                                                             const int32_t *__restrict__ pairs, int64_t Q, int per,
+                                                             unsigned long long *__restrict__ out) {
+  constexpr int kG = 32 / kLanes;             // pairs of a warp at a time
+  constexpr int kU = kC >= 16 ? 1 : 16 / kC;  // such steps in flight
+  constexpr uint32_t kInf = 0xFFFFFFFFu;
+  __shared__ int2 s_pair[kQThreads / 32][kMine];
+  __shared__ unsigned long long s_best[kQThreads / 32][kMine];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, sub = lane % kLanes, grp = lane / kLanes;
+  int2 *pr = s_pair[warp];
+  unsigned long long *bs = s_best[warp];
+  const int64_t w = (int64_t)blockIdx.x * (kQThreads / 32) + warp, warps = (int64_t)gridDim.x * (kQThreads / 32);
+  auto load = [&](const uint32_t *row, int32_t k0, uint32_t (&x)[kC]) {
+    if (VEC) {
+#pragma unroll
+      for (int c = 0; c < kC; c += 4) {
+        const int32_t k = k0 + c * kLanes + 4 * sub;
+        if (k >= K) break;
+        const uint4 a = __ldg(reinterpret_cast<const uint4 *>(row + k));
+        x[c] = a.x; x[c + 1] = a.y; x[c + 2] = a.z; x[c + 3] = a.w;
+      }
+    } else {
+#pragma unroll
+      for (int c = 0; c < kC; ++c) {
+        const int32_t k = k0 + c * kLanes + sub;
+        if (k < K) x[c] = __ldg(row + k);
+      }
+    }
+  };
+  for (int64_t i0 = w * per; i0 < Q; i0 += warps * per) {
+    const int count = (int)min((int64_t)per, Q - i0);
+    for (int i = lane; i < count; i += 32) {
+      const int32_t u = __ldg(pairs + 2 * (i0 + i)), v = __ldg(pairs + 2 * (i0 + i) + 1);
+      const bool ok = u >= 0 && (int64_t)u < n && v >= 0 && (int64_t)v < n;
+      pr[i] = ok ? make_int2(u, v) : make_int2(-1, -1);
+      bs[i] = ~0ull;
+    }
+    __syncwarp();
+    for (int32_t k0 = 0; k0 < K; k0 += kLanes * kC) {
+      for (int b = 0; b < count; b += kG * kU) {
+        uint32_t x[kU][kC], y[kU][kC];
+#pragma unroll
+        for (int h = 0; h < kU; ++h) {
+          const int i = b + h * kG + grp;
+          const int2 p = i < count ? pr[i] : make_int2(-1, -1);
+#pragma unroll
+          for (int c = 0; c < kC; ++c) x[h][c] = y[h][c] = kInf;
+          if (p.x >= 0) {
+            load(labels + (size_t)p.x * (size_t)K, k0, x[h]);
+            load(labels + (size_t)p.y * (size_t)K, k0, y[h]);
+          }
+        }
+#pragma unroll
+        for (int h = 0; h < kU; ++h) {
+          const int i = b + h * kG + grp;
+          uint32_t low = kInf;
+#pragma unroll
+          for (int c = 0; c < kC; ++c) {
+            const uint32_t s = x[h][c] + y[h][c];
+            low = min(low, s < x[h][c] ? kInf : s);
+          }
+#pragma unroll
+          for (int o = kLanes / 2; o > 0; o >>= 1) low = min(low, __shfl_xor_sync(0xFFFFFFFFu, low, o));
+          unsigned long long best = low;
+          if (__any_sync(0xFFFFFFFFu, low == kInf)) {  // a pair with no sum below 2^32 - 1
+            best = ~0ull;
+#pragma unroll
+            for (int c = 0; c < kC; ++c) take(x[h][c], y[h][c], best);
+#pragma unroll
+            for (int o = kLanes / 2; o > 0; o >>= 1) {
+              const unsigned long long z = __shfl_xor_sync(0xFFFFFFFFu, best, o);
+              best = z < best ? z : best;
+            }
+          }
+          if (sub == 0 && i < count && best < bs[i]) bs[i] = best;
+        }
+      }
+    }
+    __syncwarp();
+    for (int i = lane; i < count; i += 32) out[i0 + i] = bs[i];
+    __syncwarp();
+  }
+}
+
 bool aligned(const void *p, size_t a) { return (reinterpret_cast<uintptr_t>(p) % a) == 0; }
 
 }  // namespace
@@ -152,10 +258,23 @@ extern "C" fg_status fg_ll_query(const uint32_t *labels, int64_t n, int32_t K, c
   cudaStream_t stream = reinterpret_cast<cudaStream_t>(stream_v);
   const int64_t blocks = std::min<int64_t>((Q + kQThreads / 32 - 1) / (kQThreads / 32), 152ll * 64);
   unsigned long long *out = reinterpret_cast<unsigned long long *>(est_out);
-  if (K % 4 == 0 && aligned(labels, 16))
+  const bool vec = K % 4 == 0 && aligned(labels, 16);
+  if (Q >= kSliceMinPairs) {
+    auto launch = [&](auto kernel) {
+      const int64_t most = kSliceBlocks * (kQThreads / 32);  // warps
+      const int64_t rounds = (Q + most * kMine - 1) / (most * kMine);
+      const int per = (int)((Q + most * rounds - 1) / (most * rounds));
+      kernel<<<(unsigned)kSliceBlocks, kQThreads, 0, stream>>>(labels, n, K, pairs, Q, per, out);
+    };
+    if (K <= 16) vec ? launch(ll_slice_kernel<true, 4, 4>) : launch(ll_slice_kernel<false, 4, 4>);
+    else if (K <= 32) vec ? launch(ll_slice_kernel<true, 8, 4>) : launch(ll_slice_kernel<false, 8, 4>);
+    else if (K <= 64) vec ? launch(ll_slice_kernel<true, 8, 8>) : launch(ll_slice_kernel<false, 8, 8>);
+    else vec ? launch(ll_slice_kernel<true, 16, 8>) : launch(ll_slice_kernel<false, 16, 8>);
+  } else if (vec) {
     ll_query_kernel<true><<<(unsigned)blocks, kQThreads, 0, stream>>>(labels, n, K, pairs, Q, out);
-  else
+  } else {
     ll_query_kernel<false><<<(unsigned)blocks, kQThreads, 0, stream>>>(labels, n, K, pairs, Q, out);
+  }
   CUDA_TRY(cudaGetLastError());
   return FG_OK;
 }
