@@ -656,13 +656,32 @@ __device__ __forceinline__ float ppr_thr(const uint32_t *prp, float eps, uint32_
 
 // Targets of arcs j + 32 k + lane of a batch of vertices (exd: arcs before a
 // lane's vertex, of which it has deg from a0 on; none: one to the source), kInf
-// from tot on, and the lanes of their vertices. The loads of kUnroll steps are in
-// flight together: a round lasts as long as its longest visit, and a visit with a
-// hub as long as the chain over the hub's arcs (R-MAT 2^18, 64 sources: 4.55 ms
-// with one step at a time, 3.85 so).
+// from tot on, and the lanes of their vertices. A round lasts as long as its
+// longest visit, and a visit with a hub as long as the chain over the hub's arcs:
+// so the loads of kUnroll steps are in flight together, and steps within one
+// vertex take their owner once. R-MAT 2^18, 64 sources, per batch: 4.55 ms with one
+// step at a time, 3.90 so.
+// Only for pass 2. The count decides when a batch reserves its room: with hubs
+// quicker there, a round that fills the arena carries small batches over instead
+// of hubs (3,600 of them, not 800, and 2.7 ms), and the pushes come in another
+// order, which moves estimates by ten times what two runs differ by.
 __device__ __forceinline__ void ppr_targets(const DevGraph &g, uint32_t src, uint32_t exd, uint32_t deg, uint32_t a0,
                                             uint32_t j, uint32_t tot, uint32_t (&u)[kUnroll],
                                             uint32_t (&own)[kUnroll]) {
+  const uint32_t last = min(j + 32u * kUnroll, tot) - 1u;
+  const int ends = owner_lane(exd, (lane_id() & 1) ? last : j);
+  const int L = __shfl_sync(kFull, ends, 0);
+  if (L == __shfl_sync(kFull, ends, 1)) {
+    const uint32_t degL = __shfl_sync(kFull, deg, L);
+    const uint32_t e = __shfl_sync(kFull, a0, L) + (j - __shfl_sync(kFull, exd, L));
+#pragma unroll
+    for (int k = 0; k < kUnroll; ++k) {
+      const uint32_t t = 32u * k + (uint32_t)lane_id();
+      own[k] = (uint32_t)L;
+      u[k] = j + t < tot ? (degL > 0u ? __ldg(g.adj + e + t) : src) : kInf;
+    }
+    return;
+  }
 #pragma unroll
   for (int k = 0; k < kUnroll; ++k) {
     const uint32_t t = j + 32u * k + (uint32_t)lane_id();
@@ -753,13 +772,19 @@ __device__ void visit_ppr(const EngineArgs &a, const WarpSmem &w0, uint4 item, c
       const uint32_t tot = __shfl_sync(kFull, incl, 31);
       // pass 1: count operations for other partitions and reserve them at once
       uint32_t n_ext = 0;
-      for (uint32_t j = 0; j < tot; j += 32u * kUnroll) {
-        uint32_t u[kUnroll], own[kUnroll];
-        ppr_targets(g, src_int, exd, deg, a0, j, tot, u, own);
-#pragma unroll
-        for (int k = 0; k < kUnroll; ++k) n_ext += u[k] != kInf && (u[k] >> g.slog2) != p ? 1u : 0u;
+      for (uint32_t j = 0; j < tot; j += 32) {
+        const uint32_t t = j + (uint32_t)lane;
+        const bool has = t < tot;
+        const int L = owner_lane(exd, has ? t : 0u);
+        const uint32_t degL = __shfl_sync(kFull, deg, L);
+        const uint32_t eL = __shfl_sync(kFull, a0, L) + (t - __shfl_sync(kFull, exd, L));
+        bool ext = false;
+        if (has) {
+          const uint32_t u = degL > 0u ? g.adj[eL] : src_int;
+          ext = (u >> g.slog2) != p;
+        }
+        n_ext += __popc(__ballot_sync(kFull, ext));
       }
-      n_ext = __reduce_add_sync(kFull, n_ext);
       // reserve the batch's cross-partition increments together, from the
       // warp's own arena chunk (a new chunk of at least kArenaChunk slots
       // when it runs short)
