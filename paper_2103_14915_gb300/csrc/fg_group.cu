@@ -43,7 +43,8 @@
 // Sparse (SSSP, a vertex with at most kSparseT pending lanes): each lane
 // takes one (arc, query) pair and reads that single value. Bitwise (BFS):
 // rounds are levels, so a lane takes one arc and sets the source's frontier
-// lanes in the target's reach mask; the lanes that were new get their level.
+// lanes in the target's reach mask; the lanes that were new are pending, and get
+// their level when the vertex is visited.
 // The host orders a batch's queries before it cuts them into groups, by
 // two-hop reach, or by source position on road-like graphs, so that the
 // queries of a group advance alike.

@@ -129,12 +129,15 @@ __global__ void __launch_bounds__(kQThreads) ll_query_kernel(const uint32_t *__r
 //   n = 2^18, K = 1,023            1.61 -> 1.12  (no 16-byte loads)
 //   n = 2^18, K = 64 / 16          170 us -> 35 / 158 -> 17
 // Slices of 128 columns (64 where K ends there): with 64 and 256 the first line is
-// 0.81 and 0.92. Below kSliceMinPairs a warp per pair is the faster one:
+// 0.81 and 0.92. Of more than 2^19 vertices L2 holds less than half such a slice, and 64
+// columns are the better ones: 2^20 vertices and K = 256, 0.25 and 0.28 (a warp per pair: 0.32);
+// not where 16-byte loads are out (K = 255: 0.40 and 0.36; 0.47). Below kSliceMinPairs a warp per pair is the faster one:
 // Q = 4,000 of the first line 6.3 us and 25; 10,000 pairs of 9 columns 4.7 and 6.5;
 // 32,768 pairs 45.2 and 42.8 (K = 1,024), 65.7 and 47.6 (1,023).
 constexpr int kMine = 256;
 constexpr int64_t kSliceMinPairs = 1 << 15;
 constexpr int64_t kSliceBlocks = 152 * 4;
+constexpr int64_t kWideVertices = 1 << 19;  // 268 MB a slice of 128 columns
 
 template <bool VEC, int kLanes, int kC>
 __global__ void __launch_bounds__(kQThreads, 4) ll_slice_kernel(const uint32_t *__restrict__ labels, int64_t n, int32_t K,
@@ -268,7 +271,7 @@ extern "C" fg_status fg_ll_query(const uint32_t *labels, int64_t n, int32_t K, c
     };
     if (K <= 16) vec ? launch(ll_slice_kernel<true, 4, 4>) : launch(ll_slice_kernel<false, 4, 4>);
     else if (K <= 32) vec ? launch(ll_slice_kernel<true, 8, 4>) : launch(ll_slice_kernel<false, 8, 4>);
-    else if (K <= 64) vec ? launch(ll_slice_kernel<true, 8, 8>) : launch(ll_slice_kernel<false, 8, 8>);
+    else if (K <= 64 || (vec && n > kWideVertices)) vec ? launch(ll_slice_kernel<true, 8, 8>) : launch(ll_slice_kernel<false, 8, 8>);
     else vec ? launch(ll_slice_kernel<true, 16, 8>) : launch(ll_slice_kernel<false, 16, 8>);
   } else if (vec) {
     ll_query_kernel<true><<<(unsigned)blocks, kQThreads, 0, stream>>>(labels, n, K, pairs, Q, out);

@@ -377,7 +377,7 @@ __device__ void stream_keys(const unsigned long long *keys, int64_t count, const
 }
 
 // ---- sample -----------------------------------------------------------------
-constexpr int kBins = 4096, kBinShift = 19;     // bins of the key's FP32 bits
+constexpr int kBinsLog2 = 12, kBins = 1 << kBinsLog2, kBinShift = 19;  // bins of the key's FP32 bits
 constexpr int kChunk = 128;                     // row elements of a chunk (a float4 a lane)
 constexpr int kSampleEvery = 16;                // one chunk of so many, for rows of more than kSampleAll elements
 constexpr int64_t kSampleAll = 1 << 16;
@@ -388,81 +388,133 @@ __device__ __forceinline__ uint32_t chunk_hash(uint32_t c) {
   return c ^ (c >> 15);
 }
 
+// Encoded keys of the elements of a row's sampled chunk c, four a lane.
+template <bool VEC>
+__device__ __forceinline__ void sample_chunk(const NcpArgs &a, const float *prow, int64_t c, int every,
+                                             uint32_t (&enc)[4]) {
+  const int lane = threadIdx.x & 31;
+  const int64_t v0 = (c * every + (every > 1 ? chunk_hash((uint32_t)c) % (uint32_t)every : 0u)) * kChunk;
+  float p[4] = {0.f, 0.f, 0.f, 0.f};
+  uint32_t d[4] = {1u, 1u, 1u, 1u};
+  if (VEC) {
+    const int64_t v = v0 + 4 * lane;
+    if (v < a.n) {
+      const float4 p4 = __ldg(reinterpret_cast<const float4 *>(prow + v));
+      const uint4 d4 = __ldg(reinterpret_cast<const uint4 *>(a.deg + v));
+      p[0] = p4.x; p[1] = p4.y; p[2] = p4.z; p[3] = p4.w;
+      d[0] = d4.x; d[1] = d4.y; d[2] = d4.z; d[3] = d4.w;
+    }
+  } else {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int64_t v = v0 + e * 32 + lane;
+      if (v < a.n) {
+        p[e] = __ldg(prow + v);
+        d[e] = __ldg(a.deg + v);
+      }
+    }
+  }
+#pragma unroll
+  for (int e = 0; e < 4; ++e) enc[e] = key_enc(p[e], d[e]);
+}
+
 // Histogram of the keys of sampled chunks: block (row, part) takes chunks
 // part * kSampleChunks and on, a warp at a time.
 template <bool VEC>
 __global__ void __launch_bounds__(kThreads) ncp_sample_kernel(NcpArgs a, int parts, int64_t chunks, int every) {
   __shared__ uint32_t h[kBins];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int warp = threadIdx.x >> 5;
   const int64_t row = blockIdx.x / parts, part = blockIdx.x % parts;
   const float *prow = a.p + row * a.n;
   for (int i = threadIdx.x; i < kBins; i += kThreads) h[i] = 0u;
   __syncthreads();
   for (int64_t c = part * kSampleChunks + warp; c < chunks && c < (part + 1) * kSampleChunks; c += kWarps) {
-    const int64_t v0 = (c * every + (every > 1 ? chunk_hash((uint32_t)c) % (uint32_t)every : 0u)) * kChunk;
-    float p[4] = {0.f, 0.f, 0.f, 0.f};
-    uint32_t d[4] = {1u, 1u, 1u, 1u};
-    if (VEC) {
-      const int64_t v = v0 + 4 * lane;
-      if (v < a.n) {
-        const float4 p4 = __ldg(reinterpret_cast<const float4 *>(prow + v));
-        const uint4 d4 = __ldg(reinterpret_cast<const uint4 *>(a.deg + v));
-        p[0] = p4.x; p[1] = p4.y; p[2] = p4.z; p[3] = p4.w;
-        d[0] = d4.x; d[1] = d4.y; d[2] = d4.z; d[3] = d4.w;
-      }
-    } else {
+    uint32_t enc[4];
+    sample_chunk<VEC>(a, prow, c, every, enc);
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int64_t v = v0 + e * 32 + lane;
-        if (v < a.n) {
-          p[e] = __ldg(prow + v);
-          d[e] = __ldg(a.deg + v);
-        }
-      }
-    }
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const uint32_t enc = key_enc(p[e], d[e]);
-      if (enc) atomicAdd(&h[(enc - 1u) >> kBinShift], 1u);
-    }
+    for (int e = 0; e < 4; ++e)
+      if (enc[e]) atomicAdd(&h[(enc[e] - 1u) >> kBinShift], 1u);
   }
   __syncthreads();
   for (int i = threadIdx.x; i < kBins; i += kThreads)
     if (h[i]) atomicAdd(a.hist + row * kBins + i, h[i]);
 }
 
-// Edge of each row: the highest bin edge with at least `want` sampled keys at
-// or above it (encoded key; 1 = every key, when there are fewer).
-// A row with far more keys there than the list holds (ties) is marked for the
-// stream at once: the filter would read it for nothing.
-__global__ void __launch_bounds__(kThreads) ncp_edge_kernel(NcpArgs a, uint32_t want, int every) {
-  __shared__ uint32_t w[kWarps];
-  __shared__ uint32_t s_edge;
-  const int64_t row = blockIdx.x;
+// The highest of kBins bins (count(bin) keys each, `base` more above all of them)
+// with at least `want` keys in and above it; -1: none. Block-wide.
+template <class Count>
+__device__ int find_bin(uint32_t want, uint32_t base, uint32_t *w, int *s_bin, uint32_t *s_above, Count count) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   constexpr int kPer = kBins / kThreads;  // thread t: bins from the top, t * kPer and on
   uint32_t c[kPer], sum = 0;
 #pragma unroll
   for (int i = 0; i < kPer; ++i) {
-    c[i] = __ldcg(a.hist + row * kBins + (kBins - 1 - (tid * kPer + i)));
+    c[i] = count(kBins - 1 - (tid * kPer + i));
     sum += c[i];
   }
-  if (tid == 0) s_edge = 1u;
+  if (tid == 0) *s_bin = -1;
   const uint32_t incl = warp_prefix_incl(sum, lane);
   if (lane == 31) w[warp] = incl;
   __syncthreads();
-  uint32_t above = incl - sum;
+  uint32_t above = base + incl - sum;
   for (int i = 0; i < warp; ++i) above += w[i];
 #pragma unroll
   for (int i = 0; i < kPer; ++i) {
     if (above < want && above + c[i] >= want) {
-      s_edge = ((uint32_t)(kBins - 1 - (tid * kPer + i)) << kBinShift) + 1u;
-      if ((uint64_t)(above + c[i]) * (uint64_t)every > (uint64_t)kCap + kCap / 4) a.listed[row] = (uint32_t)kCap + 1u;
+      *s_bin = kBins - 1 - (tid * kPer + i);
+      s_above[0] = above;         // above the bin
+      s_above[1] = above + c[i];  // and with it
     }
     above += c[i];
   }
   __syncthreads();
-  if (tid == 0) a.edge[row] = s_edge;
+  return *s_bin;
+}
+
+// Edge of each row: the highest bin edge with at least `want` sampled keys at
+// or above it (encoded key; 1 = every key, when there are fewer). Where that
+// would list more keys than there is room for, as in PPR rows, whose keys crowd
+// in a few octaves, the row's sample is read again and the bin split by the next
+// twelve bits (R-MAT 2^22, PPR rows of 419 seeds: 7.4 ms without, when most rows
+// were streamed, REFINE_NOTE so). A row with too many keys even so (ties) is marked
+// for the stream at once: the filter would read it for nothing.
+template <bool VEC>
+__global__ void __launch_bounds__(kThreads) ncp_edge_kernel(NcpArgs a, uint32_t want, int64_t chunks, int every) {
+  __shared__ uint32_t h[kBins], w[kWarps], s_above[2];
+  __shared__ int s_bin;
+  const int64_t row = blockIdx.x;
+  const int bin = find_bin(want, 0u, w, &s_bin, s_above, [&](int b) { return __ldcg(a.hist + row * kBins + b); });
+  if (bin < 0) {
+    if (threadIdx.x == 0) a.edge[row] = 1u;
+    return;
+  }
+  uint32_t edge = (uint32_t)bin << kBinShift;
+  uint64_t keys = (uint64_t)s_above[1] * (uint64_t)every;
+  if (keys > (uint64_t)kCap - kCap / 8) {
+    const uint32_t above = s_above[0];
+    for (int i = threadIdx.x; i < kBins; i += kThreads) h[i] = 0u;
+    __syncthreads();
+    const float *prow = a.p + row * a.n;
+#pragma unroll 2
+    for (int64_t c = threadIdx.x >> 5; c < chunks; c += kWarps) {
+      uint32_t enc[4];
+      sample_chunk<VEC>(a, prow, c, every, enc);
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (enc[e] && (int)((enc[e] - 1u) >> kBinShift) == bin)
+          atomicAdd(&h[((enc[e] - 1u) >> (kBinShift - kBinsLog2)) & (uint32_t)(kBins - 1)], 1u);
+    }
+    __syncthreads();
+    const int fine = find_bin(want, above, w, &s_bin, s_above, [&](int b) { return h[b]; });
+    if (fine >= 0) {
+      edge |= (uint32_t)fine << (kBinShift - kBinsLog2);
+      keys = (uint64_t)s_above[1] * (uint64_t)every;
+    }
+  }
+  if (threadIdx.x == 0) {
+    a.edge[row] = edge + 1u;
+    if (keys > (uint64_t)kCap + kCap / 4) a.listed[row] = (uint32_t)kCap + 1u;
+  }
 }
 
 // ---- filter -----------------------------------------------------------------
@@ -1114,7 +1166,8 @@ extern "C" fg_status fg_ncp_sweep(fg_graph *g, const float *p, int32_t nq, int32
     e = cudaMemsetAsync(scratch, 0, 2 * b_small + b_hist, stream);
     if (vec) ncp_sample_kernel<true><<<rows * sparts, kThreads, 0, stream>>>(b, sparts, chunks, every);
     else ncp_sample_kernel<false><<<rows * sparts, kThreads, 0, stream>>>(b, sparts, chunks, every);
-    ncp_edge_kernel<<<rows, kThreads, 0, stream>>>(b, want, every);
+    if (vec) ncp_edge_kernel<true><<<rows, kThreads, 0, stream>>>(b, want, chunks, every);
+    else ncp_edge_kernel<false><<<rows, kThreads, 0, stream>>>(b, want, chunks, every);
     if (vec) ncp_filter_kernel<true><<<rows * segs, kFiltThreads, 0, stream>>>(b, segs);
     else ncp_filter_kernel<false><<<rows * segs, kFiltThreads, 0, stream>>>(b, segs);
     const unsigned streamed = (unsigned)std::min<int64_t>(rows, kStreamSlots);

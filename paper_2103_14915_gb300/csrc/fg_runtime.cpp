@@ -7,6 +7,7 @@
 #include <cstdio>
 #include <cstring>
 #include <mutex>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -172,12 +173,11 @@ static cudaError_t build_reduced(fg_graph *g, const std::vector<uint32_t> &rp, c
   for (; nh < kReduceHubs; ++nh) hubs.v[nh] = hubs.v[0];
 
   const size_t words = 2 * (size_t)((m + 63) / 64);
+  std::vector<uint32_t> keep(words);
   DevBuf table, bits;
   cudaError_t e = table.reserve(sizeof(uint32_t) * (16 * (size_t)n + kReduceRounds + 1));
   if (e == cudaSuccess) e = bits.reserve(sizeof(uint32_t) * words);
-  std::vector<uint32_t> keep;
   if (e == cudaSuccess) {
-    keep.resize(words);
     e = mark_useful_arcs(g->dg, hubs, table.as<uint32_t>(), table.as<unsigned>() + 16 * (size_t)n, bits.as<uint32_t>(),
                          nullptr);
     if (e == cudaSuccess) e = cudaMemcpy(keep.data(), bits.p, sizeof(uint32_t) * words, cudaMemcpyDeviceToHost);
@@ -463,7 +463,11 @@ extern "C" fg_status fg_graph_create_ex(int64_t n, int64_t m, const int64_t *row
     }
   }
   if (wt) {
-    const cudaError_t e = build_reduced(g, i_rp, i_adj, i_wt);
+    cudaError_t e = cudaSuccess;
+    try {
+      e = build_reduced(g, i_rp, i_adj, i_wt);
+    } catch (const std::bad_alloc &) {  // no host memory for the second copy: all arcs stay
+    }
     if (e != cudaSuccess) {
       cleanup(FG_OK);
       return fail(FG_ERR_CUDA, "marking the arcs of shortest paths: %s", cudaGetErrorString(e));
