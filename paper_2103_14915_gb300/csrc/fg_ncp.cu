@@ -108,6 +108,13 @@ __device__ __forceinline__ double dbl_dec(unsigned long long e) {
   return __longlong_as_double((long long)b);
 }
 
+// Profile: accumulate ? encode the caller's value : start from +inf (encoded).
+enum class ProfileBegin { kNone, kFresh, kAccumulate };
+__device__ __forceinline__ void profile_begin(unsigned long long *ncp, int i, bool accumulate) {
+  const double x = accumulate ? __longlong_as_double((long long)ncp[i]) : __longlong_as_double(0x7FF0000000000000ll);
+  ncp[i] = dbl_enc(x);
+}
+
 // Inclusive prefix sum within a warp.
 template <typename T>
 __device__ __forceinline__ T warp_prefix_incl(T x, int lane) {
@@ -476,13 +483,16 @@ __device__ int find_bin(uint32_t want, uint32_t base, uint32_t *w, int *s_bin, u
 // would list more keys than there is room for, as in PPR rows, whose keys crowd
 // in a few octaves, the row's sample is read again and the bin split by the next
 // twelve bits (R-MAT 2^22, PPR rows of 419 seeds: 7.4 ms without, when most rows
-// were streamed, REFINE_NOTE so). A row with too many keys even so (ties) is marked
+// were streamed, 2.2 so). A row with too many keys even so (ties) is marked
 // for the stream at once: the filter would read it for nothing.
 template <bool VEC>
-__global__ void __launch_bounds__(kThreads) ncp_edge_kernel(NcpArgs a, uint32_t want, int64_t chunks, int every) {
+__global__ void __launch_bounds__(kThreads) ncp_edge_kernel(NcpArgs a, uint32_t want, int64_t chunks, int every,
+                                                            ProfileBegin begin) {
   __shared__ uint32_t h[kBins], w[kWarps], s_above[2];
   __shared__ int s_bin;
   const int64_t row = blockIdx.x;
+  if (begin != ProfileBegin::kNone && row == 0)
+    for (int i = threadIdx.x; i < a.top; i += kThreads) profile_begin(a.ncp, i, begin == ProfileBegin::kAccumulate);
   const int bin = find_bin(want, 0u, w, &s_bin, s_above, [&](int b) { return __ldcg(a.hist + row * kBins + b); });
   if (bin < 0) {
     if (threadIdx.x == 0) a.edge[row] = 1u;
@@ -746,7 +756,7 @@ __global__ void __launch_bounds__(kThreads, 2) ncp_order_kernel(NcpArgs a, bool 
   } else {
     const Stream st = rs.on(smem);
     stream_begin(st);
-    if (row < kStreamSlots)
+    if (parts > 1 && row < kStreamSlots)
       stream_keys(a.part + (size_t)row * parts * (size_t)a.top, (int64_t)parts * a.top, st, T);
     else
       stream_part(a, row, vec, st, 0, 1);
@@ -952,10 +962,10 @@ __global__ void __launch_bounds__(kThreads) ncp_scan_kernel(NcpArgs a) {
 
 // ---- rows of few vertices -------------------------------------------------------
 // Everything for a row in one block and its shared memory, for rows of at most
-// kSmallRow vertices: what the kernels above take there is mostly their launches.
+// kSmallRow vertices, half as many more for a `top` of 512 and below: what the kernels above take there is mostly their launches.
 // 9,000 vertices, 1 row, top 300: 44 us here and 72 through them; at the line the
 // two meet (105 rows, top 4,096: 263 us here with 16,000 vertices, 255 through
-// them with 17,000).
+// them with 17,000; 1 row, top 300: 57 and 70 with 17,000, top 512: 78 and 77 with 25,000).
 constexpr int64_t kSmallRow = 1 << 14;
 constexpr size_t kSmallSmem = kInsideSmem + (size_t)kMaxTop * 4;  // and the gains
 static_assert(kSmem <= kSmallSmem, "the row is streamed in the same memory");
@@ -1004,12 +1014,9 @@ __global__ void __launch_bounds__(kThreads) ncp_small_kernel(NcpArgs a, bool vec
   scan_row(a, row, L, gain, [&](uint32_t k) { return (k + 1u < L ? m.first[k + 1u] : tot) - m.first[k]; });
 }
 
-// profile: accumulate ? encode the caller's values : start from +inf (encoded)
 __global__ void ncp_profile_begin(unsigned long long *ncp, int32_t top, int accumulate) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= top) return;
-  const double x = accumulate ? __longlong_as_double((long long)ncp[i]) : __longlong_as_double(0x7FF0000000000000ll);
-  ncp[i] = dbl_enc(x);
+  if (i < top) profile_begin(ncp, i, accumulate != 0);
 }
 
 __global__ void ncp_profile_end(unsigned long long *ncp, int32_t top) {
@@ -1097,7 +1104,8 @@ extern "C" fg_status fg_ncp_sweep(fg_graph *g, const float *p, int32_t nq, int32
   a.phi = phi_out;
   a.count = count_out;
   a.ncp = reinterpret_cast<unsigned long long *>(ncp_out);
-  if (a.ncp) {
+  const bool small = n <= kSmallRow || (n <= kSmallRow + kSmallRow / 2 && top <= 512);
+  if (a.ncp && small) {  // (else by the edge kernel)
     ncp_profile_begin<<<(top + 255) / 256, 256, 0, stream>>>(a.ncp, top, accumulate ? 1 : 0);
     CUDA_TRY(cudaGetLastError());
   }
@@ -1106,7 +1114,6 @@ extern "C" fg_status fg_ncp_sweep(fg_graph *g, const float *p, int32_t nq, int32
   // scratch (about 80 KB + 12 * top bytes a row, from the stream-ordered
   // allocator).
   constexpr int64_t kRowsPerLaunch = 1024;
-  const bool small = n <= kSmallRow;
   auto up = [](size_t b) { return (b + 255) / 256 * 256; };
   int64_t rows_max = std::min<int64_t>(nq, kRowsPerLaunch);
   size_t b_hist = 0, b_small = 0, b_list = 0, b_top = 0, b_part = 0;
@@ -1117,8 +1124,9 @@ extern "C" fg_status fg_ncp_sweep(fg_graph *g, const float *p, int32_t nq, int32
     b_small = up((size_t)rows_max * 4);
     b_list = up((size_t)rows_max * kCap * 8);
     b_top = up((size_t)rows_max * ((size_t)top + 1) * 4);
-    stream_parts = (int)std::max<int64_t>(1, std::min<int64_t>(kStreamParts, 304 / rows_max));  // two blocks an SM
-    b_part = up((size_t)std::min(rows_max, kStreamSlots) * (size_t)stream_parts * (size_t)top * 8);
+    // two blocks an SM; one part (in the order kernel) for rows that one block streams in 50 us
+    stream_parts = n <= kSampleAll ? 1 : (int)std::max<int64_t>(1, std::min<int64_t>(kStreamParts, 304 / rows_max));
+    b_part = stream_parts == 1 ? 0 : up((size_t)std::min(rows_max, kStreamSlots) * (size_t)stream_parts * (size_t)top * 8);
     const cudaError_t e0 = cudaMallocAsync(reinterpret_cast<void **>(&scratch),
                                            b_hist + 4 * b_small + b_list + 3 * b_top + b_part, stream);
     if (e0 == cudaSuccess) break;
@@ -1166,12 +1174,16 @@ extern "C" fg_status fg_ncp_sweep(fg_graph *g, const float *p, int32_t nq, int32
     e = cudaMemsetAsync(scratch, 0, 2 * b_small + b_hist, stream);
     if (vec) ncp_sample_kernel<true><<<rows * sparts, kThreads, 0, stream>>>(b, sparts, chunks, every);
     else ncp_sample_kernel<false><<<rows * sparts, kThreads, 0, stream>>>(b, sparts, chunks, every);
-    if (vec) ncp_edge_kernel<true><<<rows, kThreads, 0, stream>>>(b, want, chunks, every);
-    else ncp_edge_kernel<false><<<rows, kThreads, 0, stream>>>(b, want, chunks, every);
+    const ProfileBegin begin = !a.ncp || r0 > 0 ? ProfileBegin::kNone
+                               : accumulate     ? ProfileBegin::kAccumulate
+                                                : ProfileBegin::kFresh;
+    if (vec) ncp_edge_kernel<true><<<rows, kThreads, 0, stream>>>(b, want, chunks, every, begin);
+    else ncp_edge_kernel<false><<<rows, kThreads, 0, stream>>>(b, want, chunks, every, begin);
     if (vec) ncp_filter_kernel<true><<<rows * segs, kFiltThreads, 0, stream>>>(b, segs);
     else ncp_filter_kernel<false><<<rows * segs, kFiltThreads, 0, stream>>>(b, segs);
     const unsigned streamed = (unsigned)std::min<int64_t>(rows, kStreamSlots);
-    ncp_stream_kernel<<<streamed * stream_parts, kThreads, kSmem, stream>>>(b, vec, stream_parts);
+    if (stream_parts > 1)
+      ncp_stream_kernel<<<streamed * stream_parts, kThreads, kSmem, stream>>>(b, vec, stream_parts);
     ncp_order_kernel<<<rows, kThreads, kSmem, stream>>>(b, vec, stream_parts);
     ncp_inside_kernel<<<rows * kInsideParts, kInsideThreads, kInsideSmem, stream>>>(b, kInsideParts);
     ncp_scan_kernel<<<rows, kThreads, 0, stream>>>(b);

@@ -41,7 +41,7 @@ def rows(n, kind, nq, seed=3):
     return p
 
 
-@pytest.mark.parametrize("n", [300, 2049, 16384, 16385, 65536, 65540, 200001])
+@pytest.mark.parametrize("n", [300, 2049, 16384, 16385, 24577, 65536, 65540, 200001])
 @pytest.mark.parametrize("kind", ["spread", "sparse", "ties", "clustered"])
 def test_kept_set(n, kind):
     g = graph(n)
@@ -67,19 +67,23 @@ def test_kept_set(n, kind):
         fg.fg_graph_destroy(h)
 
 
-def test_more_rows_than_a_launch_takes():
-    g = graph(300)
+@pytest.mark.parametrize("n", [300, 24580])
+def test_more_rows_than_a_launch_takes_and_a_profile_over_two_calls(n):
+    g = graph(n)
     st, h = fg.fg_graph_create_ex(g.n, g.m, g.row_ptr, g.col, None, 0, fg.fg_default_graph_opts())
     fg.check(st)
     try:
-        p = rows(300, "sparse", 1030)
+        p = rows(n, "sparse", 1030)
         p_d = torch.from_numpy(p).to(DEV)
         order = torch.empty((1030, 50), dtype=torch.int32, device=DEV)
         phi = torch.empty((1030, 50), dtype=torch.float64, device=DEV)
-        fg.check(fg.fg_ncp_sweep(h, p_d, 1030, 50, order, phi))
+        ncp = torch.empty(50, dtype=torch.float64, device=DEV)
+        fg.check(fg.fg_ncp_sweep(h, p_d[1020:], 10, 50, None, None, None, ncp))
+        fg.check(fg.fg_ncp_sweep(h, p_d[:1029], 1029, 50, order, phi, None, ncp, True))
         fg.check(fg.fg_sync())
         ref = oracle.ncp_sweep(g, p, 50)
-        assert np.array_equal(order.cpu().numpy(), ref[0])
-        assert np.array_equal(phi.cpu().numpy(), ref[1], equal_nan=True)
+        assert np.array_equal(order[:1029].cpu().numpy(), ref[0][:1029])
+        assert np.array_equal(phi[:1029].cpu().numpy(), ref[1][:1029], equal_nan=True)
+        assert np.array_equal(ncp.cpu().numpy(), np.where(np.isnan(ref[1]), np.inf, ref[1]).min(0))
     finally:
         fg.fg_graph_destroy(h)
