@@ -16,8 +16,8 @@
 //   query               few pairs: one warp per pair reads the two K-entry
 //                       labels with 16-byte loads (K a multiple of 4) and
 //                       reduces the minimum with shuffles; 8 * K + 16 bytes per
-//                       pair. Many: the labels are taken in slices of columns
-//                       that stay in L2 while all pairs use them.
+//                       pair. Many: the labels are taken in slices of columns,
+//                       so that pairs meet in L2.
 #include <algorithm>
 #include <cstdint>
 
@@ -120,20 +120,21 @@ __global__ void __launch_bounds__(kQThreads) ll_query_kernel(const uint32_t *__r
 // Many pairs: a warp keeps up to kMine of them with their minima in shared memory
 // and takes the labels in slices of kLanes * kC columns, kLanes lanes a pair, kC
 // columns a lane, 32 words of a lane in flight. All blocks are resident and have
-// the same number of pairs, so they stay on the same few slices, which L2 holds:
-// a label is read from HBM once and not once a pair, and a pair with few columns
-// does not take a whole warp. Sums are taken in 32 bits while one of a pair's
+// the same number of pairs, so they stay on the same few slices, of which L2 holds
+// about half: of the first line's 8.6 GB of labels 4.4 come from HBM, at 78 % of its
+// peak, and a pair with few columns does not take a whole warp. Sums are taken in 32 bits while one of a pair's
 // stays below 2^32 - 1 (it is then the least of all).
-//   n = 2^18, K = 1,024, Q = 2^20  1.15 ms (7.4 TB/s) -> 0.75  (8.6 GB of labels, 1.07 GB once)
+//   n = 2^18, K = 1,024, Q = 2^20  1.15 ms (7.4 TB/s) -> 0.75  (12 TB/s; each label once: 1.07 GB)
 //   n = 2^15 (labels in L2)        0.67 -> 0.45
 //   n = 2^18, K = 1,023            1.61 -> 1.12  (no 16-byte loads)
 //   n = 2^18, K = 64 / 16          170 us -> 35 / 158 -> 17
 // Slices of 128 columns (64 where K ends there): with 64 and 256 the first line is
-// 0.81 and 0.92. Of more than 2^19 vertices L2 holds less than half such a slice, and 64
-// columns are the better ones: 2^20 vertices and K = 256, 0.25 and 0.28 (a warp per pair: 0.32);
-// not where 16-byte loads are out (K = 255: 0.40 and 0.36; 0.47). Below kSliceMinPairs a warp per pair is the faster one:
-// Q = 4,000 of the first line 6.3 us and 25; 10,000 pairs of 9 columns 4.7 and 6.5;
-// 32,768 pairs 45.2 and 42.8 (K = 1,024), 65.7 and 47.6 (1,023).
+// 0.81 and 0.92. Of more than 2^19 vertices L2 holds little of such a slice, and 64
+// columns are the better ones: 2^20 vertices and K = 256 take 0.25 ms, not 0.28 (a
+// warp per pair: 0.32); but not where 16-byte loads are out (K = 255: 0.40 and 0.36;
+// 0.47). Below kSliceMinPairs a warp per pair is the faster one: Q = 4,000 of the first
+// line 6.3 us and 25; 10,000 pairs of 9 columns 4.7 and 6.5; 32,768 pairs 45.2 and
+// 42.8 (K = 1,024), 65.7 and 47.6 (1,023).
 constexpr int kMine = 256;
 constexpr int64_t kSliceMinPairs = 1 << 15;
 constexpr int64_t kSliceBlocks = 152 * 4;
