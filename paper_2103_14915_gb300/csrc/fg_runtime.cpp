@@ -373,6 +373,7 @@ extern "C" fg_status fg_graph_create_ex(int64_t n, int64_t m, const int64_t *row
     g->hubs.release();
     g->pairs.release();
     release_reduced(g);
+    if (g->last_done) cudaEventDestroy(g->last_done);
     delete g;
     return s;
   };
@@ -477,6 +478,16 @@ extern "C" fg_status fg_graph_create_ex(int64_t n, int64_t m, const int64_t *row
   // the caller's memory is still free (lazy module loading would otherwise
   // place it at that entry point's first call)
   noalloc_prepare(dev);
+  // What was enqueued above ran on the legacy default stream, which streams
+  // created as non-blocking (the server's lanes, most callers' own) do not wait
+  // for: the graph is handed out once all of it is on the device.
+  {
+    const cudaError_t e = cudaStreamSynchronize(nullptr);
+    if (e != cudaSuccess) {
+      cleanup(FG_OK);
+      return fail(FG_ERR_CUDA, "graph upload: %s", cudaGetErrorString(e));
+    }
+  }
   *out = g;
   return FG_OK;
 }
