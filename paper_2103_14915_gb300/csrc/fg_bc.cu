@@ -89,7 +89,12 @@ __device__ __forceinline__ bool tight(uint32_t du, uint32_t wt, uint32_t dw) {
 // owner lane L, query and target; on = the arc is there and tight. (R-MAT 2^17,
 // 0.35 M arcs without those on no shortest path, 100 sources: 15.2 ms with a
 // lane per light vertex and a warp per heavy one, one arc in flight; 8.8 this way.)
+// Degrees are summed in 32 bits, at most kPassArcs of a vertex at a time: the
+// items of a warp belong to different queries, so a hub can be there 32 times,
+// and the sum of their whole degrees is not bounded by the graph's arcs.
 constexpr int kStep = 4;
+constexpr uint32_t kPassArcs = 1u << 16;
+static_assert(32ull * kPassArcs + 32ull * kStep < 1ull << 32, "the arcs of a pass are counted in 32 bits");
 
 template <class ItemAt, class Begin, class ArcFn, class End>
 __device__ __forceinline__ void walk_arcs(const BcArgs &a, int64_t count, ItemAt item_at, Begin begin, ArcFn arc_fn,
@@ -111,25 +116,31 @@ __device__ __forceinline__ void walk_arcs(const BcArgs &a, int64_t count, ItemAt
       }
     }
     begin(q, u, valid);
-    const uint32_t incl = warp_incl_scan(deg), exd = incl - deg, tot = __shfl_sync(kFull, incl, 31);
-    for (uint32_t t0 = 0; t0 < tot; t0 += 32u * kStep) {
-      uint32_t w[kStep], wt[kStep], qL[kStep], dw[kStep], dL[kStep];
-      int L[kStep];
+    for (;;) {  // the next kPassArcs of every vertex, so each one's arcs come in order
+      const uint32_t now = min(deg, kPassArcs);
+      const uint32_t incl = warp_incl_scan(now), exd = incl - now, tot = __shfl_sync(kFull, incl, 31);
+      for (uint32_t t0 = 0; t0 < tot; t0 += 32u * kStep) {
+        uint32_t w[kStep], wt[kStep], qL[kStep], dw[kStep], dL[kStep];
+        int L[kStep];
 #pragma unroll
-      for (int k = 0; k < kStep; ++k) {
-        const uint32_t t = t0 + (uint32_t)k * 32u + (uint32_t)lane;
-        const bool has = t < tot;
-        L[k] = owner_lane(exd, has ? t : 0u);
-        const uint32_t e = __shfl_sync(kFull, e0, L[k]) + (t - __shfl_sync(kFull, exd, L[k]));
-        qL[k] = __shfl_sync(kFull, q, L[k]);
-        dL[k] = __shfl_sync(kFull, du, L[k]);
-        w[k] = has ? __ldg(g.adj + e) : kInf;
-        wt[k] = has && a.weighted ? __ldg(g.wt + e) : 1u;
+        for (int k = 0; k < kStep; ++k) {
+          const uint32_t t = t0 + (uint32_t)k * 32u + (uint32_t)lane;
+          const bool has = t < tot;
+          L[k] = owner_lane(exd, has ? t : 0u);
+          const uint32_t e = __shfl_sync(kFull, e0, L[k]) + (t - __shfl_sync(kFull, exd, L[k]));
+          qL[k] = __shfl_sync(kFull, q, L[k]);
+          dL[k] = __shfl_sync(kFull, du, L[k]);
+          w[k] = has ? __ldg(g.adj + e) : kInf;
+          wt[k] = has && a.weighted ? __ldg(g.wt + e) : 1u;
+        }
+#pragma unroll
+        for (int k = 0; k < kStep; ++k) dw[k] = w[k] != kInf ? dist_of(a, qL[k], w[k]) : kInf;
+#pragma unroll
+        for (int k = 0; k < kStep; ++k) arc_fn(L[k], qL[k], w[k], tight(dL[k], wt[k], dw[k]));
       }
-#pragma unroll
-      for (int k = 0; k < kStep; ++k) dw[k] = w[k] != kInf ? dist_of(a, qL[k], w[k]) : kInf;
-#pragma unroll
-      for (int k = 0; k < kStep; ++k) arc_fn(L[k], qL[k], w[k], tight(dL[k], wt[k], dw[k]));
+      e0 += now;
+      deg -= now;
+      if (!__any_sync(kFull, deg > 0u)) break;
     }
     end(q, u, valid);
   }
