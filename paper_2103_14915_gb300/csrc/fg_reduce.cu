@@ -64,12 +64,13 @@ __global__ void __launch_bounds__(kRedThreads) reduce_round(DevGraph g, uint32_t
   if (first >= g.m) return;
   const int lane = threadIdx.x & 15;
   const unsigned mask = 0xFFFFu << (threadIdx.x & 16);
-  const uint32_t e0 = (uint32_t)first, e1 = (uint32_t)umin64(g.m, first + kRedArcs);
+  // (offsets within the piece: arc numbers near 2^32 have no room for a step past the end)
+  const uint32_t e0 = (uint32_t)first, len = (uint32_t)umin64(g.m - first, kRedArcs);
   uint32_t v = arc_owner(g.rp, g.n, e0), next = __ldg(g.rp + v + 1);
   uint32_t tv = T[(size_t)v * 16 + lane], best = tv;
   bool moved = false;
-  for (uint32_t eb = e0; eb < e1; eb += 16u) {
-    const uint32_t cnt = e1 - eb < 16u ? e1 - eb : 16u;
+  for (uint32_t o = 0; o < len; o += 16u) {
+    const uint32_t eb = e0 + o, cnt = min(len - o, 16u);
     const uint32_t xa = (uint32_t)lane < cnt ? __ldg(g.adj + eb + lane) : 0u;
     const uint32_t wa = (uint32_t)lane < cnt ? __ldg(g.wt + eb + lane) : 0u;
     uint32_t t[16];
@@ -117,12 +118,12 @@ __global__ void __launch_bounds__(kRedThreads) reduce_mark(DevGraph g, const uin
   if (first >= g.m) return;
   const int lane = threadIdx.x & 7;
   const unsigned mask = 0xFFu << (threadIdx.x & 24);
-  const uint32_t e0 = (uint32_t)first, e1 = (uint32_t)umin64(g.m, first + kMarkArcs);
+  const uint32_t e0 = (uint32_t)first, len = (uint32_t)umin64(g.m - first, kMarkArcs);
   uint32_t v = arc_owner(g.rp, g.n, e0), next = __ldg(g.rp + v + 1);
   uint32_t rv = __ldg(T + (size_t)v * 16 + lane);
   uint64_t keep = 0ull;
-  for (uint32_t eb = e0; eb < e1; eb += 8u) {
-    const uint32_t cnt = e1 - eb < 8u ? e1 - eb : 8u;
+  for (uint32_t o = 0; o < len; o += 8u) {
+    const uint32_t eb = e0 + o, cnt = min(len - o, 8u);
     const uint32_t xa = (uint32_t)lane < cnt ? __ldg(g.adj + eb + lane) : 0u;
     const uint32_t wa = (uint32_t)lane < cnt ? __ldg(g.wt + eb + lane) : 0u;
     uint32_t f[8];
@@ -144,7 +145,7 @@ __global__ void __launch_bounds__(kRedThreads) reduce_mark(DevGraph g, const uin
       s = min(s, __shfl_xor_sync(mask, s, 1, 8));
       s = min(s, __shfl_xor_sync(mask, s, 2, 8));
       s = min(s, __shfl_xor_sync(mask, s, 4, 8));
-      if (s >= w) keep |= 1ull << (eb - e0 + (uint32_t)j);
+      if (s >= w) keep |= 1ull << (o + (uint32_t)j);
     }
   }
   if (lane == 0) bits[grp] = make_uint2((uint32_t)keep, (uint32_t)(keep >> 32));
