@@ -140,7 +140,7 @@ __device__ __forceinline__ void walk_arcs(const BcArgs &a, int64_t count, ItemAt
       }
       e0 += now;
       deg -= now;
-      if (!__any_sync(kFull, deg > 0u)) break;
+      if (g.max_deg <= kPassArcs || !__any_sync(kFull, deg > 0u)) break;
     }
     end(q, u, valid);
   }
@@ -189,7 +189,7 @@ __device__ __forceinline__ double dep_term(double su, double sw, double dw) {
   return __dmul_rn(__ddiv_rn(su, sw), __dadd_rn(1.0, dw));
 }
 
-__global__ void __launch_bounds__(kBcThreads) bc_kernel(BcArgs a) {
+__global__ void __launch_bounds__(kBcThreads, 3) bc_kernel(BcArgs a) {
   const int64_t n = a.g.n;
   const int64_t nthreads = (int64_t)gridDim.x * blockDim.x;
   const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
