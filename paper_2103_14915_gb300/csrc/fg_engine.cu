@@ -234,6 +234,12 @@ __device__ __forceinline__ bool arcs_in_range(const DevGraph &g, uint32_t e0, ui
   return (uint64_t)e0 + deg <= g.m;
 }
 
+// The arc after the `step` from j on, or tot: tot may be any number below 2^32,
+// so j + step must not pass it.
+__device__ __forceinline__ uint32_t next_arcs(uint32_t j, uint32_t tot, uint32_t step) {
+  return tot - j > step ? j + step : tot;
+}
+
 // The visit's queue: positions head .. tail - 1 of the ring (modulo S).
 struct Queue {
   uint32_t head = 0, tail = 0;  // the same in every lane
@@ -571,16 +577,17 @@ __device__ void visit_dist(const EngineArgs &a, const DistSmem &w, uint4 item, u
       const uint32_t exd = incl - deg;
       const uint32_t tot = __shfl_sync(kFull, incl, 31);
       arcs += deg;
-      for (uint32_t j = 0; j < tot; j += 32u * kUnroll) {
+      for (uint32_t j = 0; j < tot; j = next_arcs(j, tot, 32u * kUnroll)) {
+        const uint32_t left = tot - j;
         uint32_t u[kUnroll], wt[kUnroll], own[kUnroll];
 #pragma unroll
         for (int k = 0; k < kUnroll; ++k) {
           u[k] = kInf;
           wt[k] = 1u;
           own[k] = 0u;
-          if (j + 32u * (uint32_t)k < tot) {  // warp-uniform
+          if (32u * (uint32_t)k < left) {  // warp-uniform
             const uint32_t t = j + 32u * (uint32_t)k + (uint32_t)lane;
-            const bool has = t < tot;
+            const bool has = 32u * (uint32_t)k + (uint32_t)lane < left;
             const int L = owner_lane(exd, has ? t : 0u);
             const uint32_t eL = __shfl_sync(kFull, a0, L) + (t - __shfl_sync(kFull, exd, L));
             own[k] = (uint32_t)L;
@@ -656,7 +663,7 @@ __device__ __forceinline__ float ppr_thr(const uint32_t *prp, float eps, uint32_
 
 // Targets of arcs j + 32 k + lane of a batch of vertices (exd: arcs before a
 // lane's vertex, of which it has deg from a0 on; none: one to the source), kInf
-// from tot on, and the lanes of their vertices. A round lasts as long as its
+// beyond the `left` that there are from j on, and the lanes of their vertices. A round lasts as long as its
 // longest visit, and a visit with a hub as long as the chain over the hub's arcs:
 // so the loads of kUnroll steps are in flight together, and steps within one
 // vertex take their owner once. R-MAT 2^18, 64 sources, per batch: 4.55 ms with one
@@ -666,9 +673,9 @@ __device__ __forceinline__ float ppr_thr(const uint32_t *prp, float eps, uint32_
 // of hubs (3,600 of them, not 800, and 2.7 ms), and the pushes come in another
 // order, which moves estimates by ten times what two runs differ by.
 __device__ __forceinline__ void ppr_targets(const DevGraph &g, uint32_t src, uint32_t exd, uint32_t deg, uint32_t a0,
-                                            uint32_t j, uint32_t tot, uint32_t (&u)[kUnroll],
+                                            uint32_t j, uint32_t left, uint32_t (&u)[kUnroll],
                                             uint32_t (&own)[kUnroll]) {
-  const uint32_t last = min(j + 32u * kUnroll, tot) - 1u;
+  const uint32_t last = j + (min(32u * kUnroll, left) - 1u);
   const int ends = owner_lane(exd, (lane_id() & 1) ? last : j);
   const int L = __shfl_sync(kFull, ends, 0);
   if (L == __shfl_sync(kFull, ends, 1)) {
@@ -678,17 +685,18 @@ __device__ __forceinline__ void ppr_targets(const DevGraph &g, uint32_t src, uin
     for (int k = 0; k < kUnroll; ++k) {
       const uint32_t t = 32u * k + (uint32_t)lane_id();
       own[k] = (uint32_t)L;
-      u[k] = j + t < tot ? (degL > 0u ? __ldg(g.adj + e + t) : src) : kInf;
+      u[k] = t < left ? (degL > 0u ? __ldg(g.adj + e + t) : src) : kInf;
     }
     return;
   }
 #pragma unroll
   for (int k = 0; k < kUnroll; ++k) {
     const uint32_t t = j + 32u * k + (uint32_t)lane_id();
-    own[k] = (uint32_t)owner_lane(exd, t < tot ? t : 0u);
+    const bool has = 32u * k + (uint32_t)lane_id() < left;
+    own[k] = (uint32_t)owner_lane(exd, has ? t : 0u);
     const uint32_t degL = __shfl_sync(kFull, deg, (int)own[k]);
     const uint32_t e = __shfl_sync(kFull, a0, (int)own[k]) + (t - __shfl_sync(kFull, exd, (int)own[k]));
-    u[k] = t < tot ? (degL > 0u ? __ldg(g.adj + e) : src) : kInf;
+    u[k] = has ? (degL > 0u ? __ldg(g.adj + e) : src) : kInf;
   }
 }
 
@@ -828,9 +836,9 @@ __device__ void visit_ppr(const EngineArgs &a, const WarpSmem &w0, uint4 item, c
       vis_edges += tot;
       // pass 2: spread (1 - alpha) rho
       uint32_t run = 0;
-      for (uint32_t j = 0; j < tot; j += 32u * kUnroll) {
+      for (uint32_t j = 0; j < tot; j = next_arcs(j, tot, 32u * kUnroll)) {
         uint32_t u[kUnroll], own[kUnroll];
-        ppr_targets(g, src_int, exd, deg, a0, j, tot, u, own);
+        ppr_targets(g, src_int, exd, deg, a0, j, tot - j, u, own);
 #pragma unroll
         for (int k = 0; k < kUnroll; ++k) {
           const float inc = __shfl_sync(kFull, inc_l, (int)own[k]);
