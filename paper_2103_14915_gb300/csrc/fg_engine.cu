@@ -472,7 +472,11 @@ __device__ void visit_dist(const EngineArgs &a, const DistSmem &w, uint4 item, u
   }
 
   const bool a_yields = a.yield_edges != 0;
-  uint32_t steps = 0, arcs = 0;  // arcs: of this lane
+  uint32_t steps = 0;
+  uint32_t arcs = 0;        // PAIRS: of this lane, at most four a step
+  uint64_t warp_arcs = 0;   // else: of the warp; hubs taken again and again pass 2^32
+  auto scanned = [&]() -> uint64_t { return PAIRS ? (uint64_t)__reduce_add_sync(kFull, arcs) : warp_arcs; };
+  static_assert(32ull * 4ull * kMaxVisitSteps < 1ull << 32, "the arcs of a PAIRS visit are counted in 32 bits");
   for (;;) {
     // everything but taking a step stands behind one branch
     if ((qu.head == qu.tail) | (++steps % 256u == 0u) | a_yields | arena_pressed(a, sl.seen)) {
@@ -518,7 +522,7 @@ __device__ void visit_dist(const EngineArgs &a, const DistSmem &w, uint4 item, u
         continue;
       }
       // yield heuristic 1, or arena pressure: leave the rest to a later visit
-      if ((a_yields && __reduce_add_sync(kFull, arcs) >= a.yield_edges) || arena_pressed(a, sl.seen)) break;
+      if ((a_yields && scanned() >= a.yield_edges) || arena_pressed(a, sl.seen)) break;
     }
     const uint32_t F = min(qu.tail - qu.head, PAIRS ? 16u : 32u);
     // A vertex leaves the queue before its value is read, so that a later fall
@@ -576,7 +580,7 @@ __device__ void visit_dist(const EngineArgs &a, const DistSmem &w, uint4 item, u
       const uint32_t incl = warp_incl_scan(deg);
       const uint32_t exd = incl - deg;
       const uint32_t tot = __shfl_sync(kFull, incl, 31);
-      arcs += deg;
+      warp_arcs += tot;
       for (uint32_t j = 0; j < tot; j = next_arcs(j, tot, 32u * kUnroll)) {
         const uint32_t left = tot - j;
         uint32_t u[kUnroll], wt[kUnroll], own[kUnroll];
@@ -614,7 +618,7 @@ __device__ void visit_dist(const EngineArgs &a, const DistSmem &w, uint4 item, u
     }
     __syncwarp();  // the queue's new entries are read by the next step
   }
-  ctr.edges += __reduce_add_sync(kFull, arcs);
+  ctr.edges += scanned();
   if (xl.n > 0u) ext_send(a, w, xl, xl.n, q, ctr, sl);
   __syncwarp();
 
