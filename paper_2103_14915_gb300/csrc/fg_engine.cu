@@ -471,7 +471,12 @@ __device__ void visit_dist(const EngineArgs &a, const DistSmem &w, uint4 item, u
     __syncwarp();
   }
 
+  // Yield heuristic 1 is asked each time the vertices that were queued when it
+  // was asked last have been taken: a step takes 16 or 32 of them, and a visit
+  // that stops among them leaves the rest of a frontier to another round (256^2
+  // grid, 64 SSSP sources, yield_edges 64: 115 ms asked every step, 29 so).
   const bool a_yields = a.yield_edges != 0;
+  uint32_t turn = 0;  // queue position
   uint32_t steps = 0;
   uint32_t arcs = 0;        // PAIRS: of this lane, at most four a step
   uint64_t warp_arcs = 0;   // else: of the warp; hubs taken again and again pass 2^32
@@ -479,7 +484,8 @@ __device__ void visit_dist(const EngineArgs &a, const DistSmem &w, uint4 item, u
   static_assert(32ull * 4ull * kMaxVisitSteps < 1ull << 32, "the arcs of a PAIRS visit are counted in 32 bits");
   for (;;) {
     // everything but taking a step stands behind one branch
-    if ((qu.head == qu.tail) | (++steps % 256u == 0u) | a_yields | arena_pressed(a, sl.seen)) {
+    if ((qu.head == qu.tail) | (++steps % 256u == 0u) | (a_yields & ((int32_t)(qu.head - turn) >= 0)) |
+        arena_pressed(a, sl.seen)) {
       // bounded loop: a visit can never spin forever
       if (steps > kMaxVisitSteps) {
         raise_status(a.ctrl, FG_ERR_TIMEOUT, kSiteVisit);
@@ -522,7 +528,11 @@ __device__ void visit_dist(const EngineArgs &a, const DistSmem &w, uint4 item, u
         continue;
       }
       // yield heuristic 1, or arena pressure: leave the rest to a later visit
-      if ((a_yields && scanned() >= a.yield_edges) || arena_pressed(a, sl.seen)) break;
+      if (a_yields && (int32_t)(qu.head - turn) >= 0) {
+        if (scanned() >= a.yield_edges) break;
+        turn = qu.tail;
+      }
+      if (arena_pressed(a, sl.seen)) break;
     }
     const uint32_t F = min(qu.tail - qu.head, PAIRS ? 16u : 32u);
     // A vertex leaves the queue before its value is read, so that a later fall
