@@ -25,6 +25,7 @@
 // slice of that partition has a single writer (the atomic-free consolidation
 // of Sec. 4.2, here at warp granularity). Operations to other partitions are
 // filtered by a plain read of the target's committed value (SSSP/BFS).
+#include <algorithm>
 #include <cstdio>
 
 #include "fg_device.cuh"
@@ -89,7 +90,10 @@ __host__ __device__ inline size_t warp_smem_words(bool ppr, int S) {
 // of the arena at a time, so the device-wide cursor is touched once per chunk
 // rather than once per append (a returning atomic on one address that every
 // warp of the grid shares). Reserved slots a warp does not fill become holes
-// (kInvalidKey) that SCATTER skips. Without ArenaSlots (seeding), each call
+// (kInvalidKey) that SCATTER skips. An arena too small for a few chunks of every
+// busy warp is reserved slot by slot (a.arena_chunk, launch_engine): a visit that
+// sends five operations must not keep 59 others from theirs, who would take the
+// same vertices up again in the next round. Without ArenaSlots (seeding), each call
 // reserves exactly what it appends.
 // ---------------------------------------------------------------------------
 struct ArenaSlots {
@@ -123,10 +127,11 @@ __device__ __forceinline__ bool emit_ops(const EngineArgs &a, bool has, uint32_t
   if (sl != nullptr) {
     if (sl->pos + n > sl->end) {
       release_slots(a, *sl);
-      if (lane == 0) base = atomicAdd(&a.ctrl->e_cursor, (unsigned long long)kArenaChunk);
+      const unsigned take = max(n, a.arena_chunk);
+      if (lane == 0) base = atomicAdd(&a.ctrl->e_cursor, (unsigned long long)take);
       base = __shfl_sync(kFull, base, 0);
       sl->pos = base;
-      sl->end = base + kArenaChunk;
+      sl->end = base + take;
       sl->seen = sl->end;
     }
     base = sl->pos;
@@ -1486,6 +1491,12 @@ cudaError_t engine_grid_size(int qtype, bool pairs, int S, int *blocks, int *thr
 
 cudaError_t launch_engine(const EngineArgs &a, int blocks, int threads, size_t smem, cudaStream_t s) {
   EngineArgs copy = a;
+  // SSSP / BFS: whole chunks while the arena holds four of every warp that can be
+  // busy. A visit sends what leaves its partition at its end, so with fewer the
+  // first visits to end would take the arena (64 sources, 256^2 grid: 512 slots
+  // 4.2 s with chunks, 1.8 without; 4,096 slots 490 and 207 ms; 32,768 slots 102 and 46).
+  const uint64_t busy = std::min<uint64_t>((uint64_t)a.g.nparts * (uint64_t)a.nq, (uint64_t)blocks * kWarps);
+  copy.arena_chunk = a.e_cap < 4ull * kArenaChunk * busy ? 1u : kArenaChunk;
   void *args[] = {(void *)&copy};
   return cudaLaunchCooperativeKernel(engine_fn(a.qtype, a.g.pairs != nullptr), dim3(blocks), dim3(threads), args, smem, s);
 }

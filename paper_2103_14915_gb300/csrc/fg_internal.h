@@ -107,6 +107,7 @@ struct EngineArgs {
   uint2 *e_op = nullptr;
   uint2 *b_op = nullptr;
   uint64_t e_cap = 0;
+  uint32_t arena_chunk = 1;  // SSSP / BFS: arena slots a warp reserves at once, at least (launch_engine)
   Ctrl *ctrl = nullptr;
   // options
   uint32_t delta = 0, bucket = 0, sched = 0, sched_window = 0;
