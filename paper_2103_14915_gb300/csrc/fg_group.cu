@@ -139,15 +139,13 @@ __host__ __device__ __forceinline__ uint32_t overflow_limit(const DevGraph &g) {
 
 // A vertex's final value on a graph that SSSP runs on without its arcs that
 // lie on no shortest path: reports the overflow that one of the vertex's arcs,
-// left out or not, makes (the relaxations see only the arcs that are in).
+// left out or not, makes (the relaxations see only the arcs that are in). Its
+// heaviest arc decides, so one read tells: with one heavy arc in the graph all
+// values beyond it are above the limit, and a look at every arc of a hub by one
+// thread took 275 ms (hub of 2^20 arcs, 64 queries behind the arc) of a batch of 1.6.
 __device__ __forceinline__ void check_all_arcs(const GroupArgs &a, uint32_t lim, uint32_t v, uint32_t d) {
   if (d == kInf || d < lim) return;
-  const uint32_t e1 = a.all_rp[v + 1];
-  for (uint32_t e = a.all_rp[v]; e < e1; ++e)
-    if ((uint64_t)d + (uint64_t)a.all_wt[e] >= (uint64_t)kInf) {
-      atomicCAS(&a.ctrl->status, 0, (int)FG_ERR_OVERFLOW);
-      return;
-    }
+  if ((uint64_t)d + (uint64_t)__ldg(a.most_wt + v) >= (uint64_t)kInf) atomicCAS(&a.ctrl->status, 0, (int)FG_ERR_OVERFLOW);
 }
 
 __host__ __device__ constexpr int ilog2c(int x) { return x <= 1 ? 0 : 1 + ilog2c(x / 2); }
@@ -443,7 +441,7 @@ __global__ void __launch_bounds__(kGThreads, 3) group_kernel(GroupArgs a) {
             uint32_t *pv = Dg + (v << LG) + (uint64_t)gg;
             const uint32_t x = __ldcg(pv);
             a.res[((uint64_t)grp * (uint64_t)Gq + (uint64_t)gg) * (uint64_t)G.n + o] = x;
-            if (QT == Q_SSSP && a.all_rp != nullptr) check_all_arcs(a, ovf_lim, (uint32_t)v, x);
+            if (QT == Q_SSSP && a.most_wt != nullptr) check_all_arcs(a, ovf_lim, (uint32_t)v, x);
             *pv = kInf;  // the lane starts over for its next request
           }
         }
@@ -1079,7 +1077,7 @@ __global__ void __launch_bounds__(256) group_out_kernel(GroupArgs a, uint32_t *o
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
         t[q + c][vl] = y[c];
-        if (a.all_rp != nullptr) check_all_arcs(a, lim, (uint32_t)(v0 + vl), y[c]);
+        if (a.most_wt != nullptr) check_all_arcs(a, lim, (uint32_t)(v0 + vl), y[c]);
       }
     }
   }

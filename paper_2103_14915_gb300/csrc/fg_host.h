@@ -158,6 +158,7 @@ struct fg_graph {
   // SSSP in the group engine: the graph without the arcs that lie on no
   // shortest path (fg_reduce.cu), when enough of them were found at creation
   fg::DevBuf s_rp, s_adj, s_wt, s_hubs;
+  fg::DevBuf s_most;               // heaviest arc of a vertex in the whole graph, where a sum can overflow
   fg::DevGraph s_dg;
   int32_t s_nhubs = 0;
   bool reduced = false;

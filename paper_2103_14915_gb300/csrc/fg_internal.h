@@ -153,8 +153,9 @@ struct GroupArgs {
   uint32_t *seen = nullptr;       // [slots] sequence number of each slot's current request
   uint32_t *gact = nullptr;       // [2][ngroups] lanes with pending work in the round of that parity
   // SSSP on a graph without its arcs that lie on no shortest path (g is then
-  // that graph): the whole graph's arcs, for the overflow test alone
-  const uint32_t *all_rp = nullptr, *all_wt = nullptr;
+  // that graph): the heaviest arc of every vertex in the whole graph, for the
+  // overflow test (null where no sum of the graph can reach 2^32 - 1)
+  const uint32_t *most_wt = nullptr;
   uint32_t check_staging = 0;     // 1: compare every staged word with global memory (self-test)
   uint32_t init = 0;              // 1: first launch on this state: fill it before the first round
   uint32_t round0 = 0;            // number of the first round (its parity selects the mask halves)

@@ -136,7 +136,7 @@ static fg_status validate_csr(int64_t n, int64_t m, const int64_t *row_ptr, cons
 }
 
 static void release_reduced(fg_graph *g) {
-  g->s_rp.release(); g->s_adj.release(); g->s_wt.release(); g->s_hubs.release();
+  g->s_rp.release(); g->s_adj.release(); g->s_wt.release(); g->s_hubs.release(); g->s_most.release();
   g->reduced = false;
 }
 
@@ -217,12 +217,24 @@ static cudaError_t build_reduced(fg_graph *g, const std::vector<uint32_t> &rp, c
     if (deg > kHubMin) hub_list.push_back((uint32_t)v);
   }
   r_rp[(size_t)n] = (uint32_t)k;
+  // the heaviest arc of every vertex, left out or not, for the overflow test;
+  // where no path of n arcs reaches 2^32 - 1 there is nothing to test
+  std::vector<uint32_t> most;
+  if ((uint64_t)n * (uint64_t)g->max_weight >= 0xFFFFFFFFull) {
+    most.resize((size_t)n);
+    for (int64_t v = 0; v < n; ++v) {
+      uint32_t x = 0;
+      for (uint64_t a = rp[(size_t)v]; a < rp[(size_t)v + 1]; ++a) x = std::max(x, wt[(size_t)a]);
+      most[(size_t)v] = x;
+    }
+  }
 
   const size_t rp_elems = (size_t)g->nparts * (size_t)g->S + 64, arc_elems = (size_t)kept + 64;
   e = g->s_rp.reserve(sizeof(uint32_t) * rp_elems);
   if (e == cudaSuccess) e = g->s_adj.reserve(sizeof(uint32_t) * arc_elems);
   if (e == cudaSuccess) e = g->s_wt.reserve(sizeof(uint32_t) * arc_elems);
   if (e == cudaSuccess && !hub_list.empty()) e = g->s_hubs.reserve(sizeof(uint32_t) * hub_list.size());
+  if (e == cudaSuccess && !most.empty()) e = g->s_most.reserve(sizeof(uint32_t) * most.size());
   if (e == cudaErrorMemoryAllocation) {
     (void)cudaGetLastError();
     release_reduced(g);
@@ -238,6 +250,7 @@ static cudaError_t build_reduced(fg_graph *g, const std::vector<uint32_t> &rp, c
   put(g->s_adj, r_adj, arc_elems);
   put(g->s_wt, r_wt, arc_elems);
   if (!hub_list.empty()) put(g->s_hubs, hub_list, hub_list.size());
+  if (!most.empty()) put(g->s_most, most, most.size());
   if (e != cudaSuccess) return e;
   g->s_dg = g->dg;
   g->s_dg.m = kept;
@@ -247,7 +260,7 @@ static cudaError_t build_reduced(fg_graph *g, const std::vector<uint32_t> &rp, c
   g->s_dg.wt = g->s_wt.as<uint32_t>();
   g->s_nhubs = (int32_t)hub_list.size();
   g->reduced = true;
-  g->graph_bytes += sizeof(uint32_t) * ((size_t)n + 1 + 2 * (size_t)kept);
+  g->graph_bytes += sizeof(uint32_t) * ((size_t)n + 1 + 2 * (size_t)kept + most.size());
   return cudaSuccess;
 }
 
@@ -1130,8 +1143,7 @@ void set_group_graph(const fg_graph *g, int qtype, GroupArgs &a) {
   a.g = red ? g->s_dg : g->dg;
   a.nhubs = red ? g->s_nhubs : g->nhubs;
   a.hubs = a.nhubs ? (red ? g->s_hubs : g->hubs).as<uint32_t>() : nullptr;
-  a.all_rp = red ? g->dg.rp : nullptr;
-  a.all_wt = red ? g->dg.wt : nullptr;
+  a.most_wt = red ? g->s_most.as<uint32_t>() : nullptr;
 }
 
 fg_status report_error(fg_status s, const char *msg) {
