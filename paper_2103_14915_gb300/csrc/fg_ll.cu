@@ -133,11 +133,22 @@ __global__ void __launch_bounds__(kQThreads) ll_query_kernel(const uint32_t *__r
 // columns are the better ones: 2^20 vertices and K = 256 take 0.25 ms, not 0.28 (a
 // warp per pair: 0.32); but not where 16-byte loads are out (K = 255: 0.40 and 0.36;
 // 0.47). Below kSliceMinPairs a warp per pair is the faster one: Q = 4,000 of the first
-// line 6.3 us and 25; 10,000 pairs of 9 columns 4.7 and 6.5; 32,768 pairs 45.2 and
-// 42.8 (K = 1,024), 65.7 and 47.6 (1,023).
+// line 6.3 us and 25; 10,000 pairs of 9 columns 4.7 and 6.5; 32,768 pairs of 64 columns
+// 19 and 16. Where L2 holds all labels (kL2Labels) slices win nothing by what they
+// find there, and a warp streams a wide row without a vote and a shuffle tree every
+// 128 columns: such rows of 16-byte loads, 2^12 vertices, take a warp per pair up to
+// kSliceWidePairs pairs (512 columns: 2^15 pairs 24 us, 26 in slices; 2^16 35 and 36;
+// 2^17 54 and 52), and beyond 2 * kWideRow columns for any number (1,024 columns: 2^16
+// pairs 47 and 56, 2^20 522 and 562; 4,096 columns 134 and 174 for 2^16; without 16-byte
+// loads, 767 columns, 2^20 552 and 474). The sizes do not tell of pairs that keep to a few vertices of a large
+// graph: they are in L2 either way, and cost up to a third more in slices (64 of
+// 2^18 vertices, 1,024 columns: 2^15 pairs 31 and 37 us, 2^20 518 and 537).
 constexpr int kMine = 256;
 constexpr int64_t kSliceMinPairs = 1 << 15;
 constexpr int64_t kSliceBlocks = 152 * 4;
+constexpr int32_t kWideRow = 256;
+constexpr int64_t kSliceWidePairs = 1 << 16;
+constexpr int64_t kL2Labels = 100ll << 20;  // (64 MB of labels are read at L2's rate, 134 MB are not)
 constexpr int64_t kWideVertices = 1 << 19;  // 268 MB a slice of 128 columns
 
 template <bool VEC, int kLanes, int kC>
@@ -204,15 +215,23 @@ __global__ void __launch_bounds__(kQThreads, 4) ll_slice_kernel(const uint32_t *
           }
 #pragma unroll
           for (int o = kLanes / 2; o > 0; o >>= 1) low = min(low, __shfl_xor_sync(0xFFFFFFFFu, low, o));
-          unsigned long long best = low;
-          if (__any_sync(0xFFFFFFFFu, low == kInf)) {  // a pair with no sum below 2^32 - 1
-            best = ~0ull;
+          // No sum below 2^32 - 1: mostly a pair that no landmark of the slice
+          // reaches (or no pair at all), with nothing to take. Only if a column
+          // has two finite distances is their sum one of more than 32 bits.
+          unsigned long long best = low == kInf ? ~0ull : low;
+          if (__any_sync(0xFFFFFFFFu, low == kInf)) {
+            uint32_t both = kInf;
 #pragma unroll
-            for (int c = 0; c < kC; ++c) take(x[h][c], y[h][c], best);
+            for (int c = 0; c < kC; ++c) both = min(both, max(x[h][c], y[h][c]));
+            if (__any_sync(0xFFFFFFFFu, low == kInf && both != kInf)) {
+              best = ~0ull;
 #pragma unroll
-            for (int o = kLanes / 2; o > 0; o >>= 1) {
-              const unsigned long long z = __shfl_xor_sync(0xFFFFFFFFu, best, o);
-              best = z < best ? z : best;
+              for (int c = 0; c < kC; ++c) take(x[h][c], y[h][c], best);
+#pragma unroll
+              for (int o = kLanes / 2; o > 0; o >>= 1) {
+                const unsigned long long z = __shfl_xor_sync(0xFFFFFFFFu, best, o);
+                best = z < best ? z : best;
+              }
             }
           }
           if (sub == 0 && i < count && best < bs[i]) bs[i] = best;
@@ -263,7 +282,9 @@ extern "C" fg_status fg_ll_query(const uint32_t *labels, int64_t n, int32_t K, c
   const int64_t blocks = std::min<int64_t>((Q + kQThreads / 32 - 1) / (kQThreads / 32), 152ll * 64);
   unsigned long long *out = reinterpret_cast<unsigned long long *>(est_out);
   const bool vec = K % 4 == 0 && aligned(labels, 16);
-  if (Q >= kSliceMinPairs) {
+  const bool wide_in_l2 = vec && K > kWideRow && n * (int64_t)K * 4 <= kL2Labels;
+  const bool sliced = Q >= kSliceMinPairs && !(wide_in_l2 && (K > 2 * kWideRow || Q < kSliceWidePairs));
+  if (sliced) {
     auto launch = [&](auto kernel) {
       const int64_t most = kSliceBlocks * (kQThreads / 32);  // warps
       const int64_t rounds = (Q + most * kMine - 1) / (most * kMine);
