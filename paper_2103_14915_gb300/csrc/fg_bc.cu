@@ -36,7 +36,6 @@ namespace fg {
 namespace {
 
 constexpr int kBcThreads = 256;
-constexpr uint32_t kRoadDegree = 64;  // max out-degree up to which a graph takes one block per source
 constexpr double kExactLimit = 9007199254740992.0;  // 2^53
 
 // Counters of one launch (zeroed before it). Wave t appends the vertices it

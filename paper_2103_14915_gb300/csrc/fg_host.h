@@ -142,6 +142,7 @@ struct fg_graph {
   size_t engine_smem = 0;
   int engine_qtype = -1;
   uint32_t max_degree = 0;
+  uint64_t hub_arcs = 0;           // arcs of the vertices with more than kRoadDegree
   double mean_weight = 1.0;        // mean arc weight (1 when unweighted)
   uint32_t min_weight = 0;         // smallest arc weight (0 when unweighted)
   uint32_t max_weight = 0;         // largest arc weight (0 when unweighted)
@@ -170,6 +171,7 @@ struct fg_graph {
 
 namespace fg {
 
+constexpr uint32_t kRoadDegree = 64;  // out-degrees up to which a vertex may be a road crossing
 constexpr uint32_t kHubMin = 512;     // group engine: vertices with more arcs are hubs
 constexpr uint32_t kHubChunk = 4096;  // group engine: arcs per hub chunk
 
@@ -179,8 +181,9 @@ bool groups_by_default(const fg_graph *g);
 // The query group that fg_opts.group = 0 resolves to for a batch of nq queries
 // of one kind: where groups_by_default, 64, or 32 for SSSP under a window, or 8
 // or 16 for SSSP with little state (the smallest of 8, 16, 32, 64 that holds a
-// smaller batch, and one that fits shared memory); else 1.
-int auto_group_size(const fg_graph *g, int qtype, int64_t nq, bool windowed);
+// smaller batch, and one that fits shared memory); else 1, as for SSSP with a
+// window or a delta on a graph of few partitions and few arcs at its hubs.
+int auto_group_size(const fg_graph *g, int qtype, int64_t nq, bool windowed, bool delayed);
 
 // The graph and hubs a group-engine launch of this query kind runs on.
 void set_group_graph(const fg_graph *g, int qtype, GroupArgs &a);

@@ -429,6 +429,7 @@ extern "C" fg_status fg_graph_create_ex(int64_t n, int64_t m, const int64_t *row
   for (int64_t v = 0; v < n; ++v) {
     const uint32_t deg = i_rp[(size_t)v + 1] - i_rp[(size_t)v];
     g->max_degree = std::max(g->max_degree, deg);
+    if (deg > kRoadDegree) g->hub_arcs += deg;
     if (deg > kHubMin) {
       hubs.push_back((uint32_t)v);
       g->hub_chunks += (deg + kHubChunk - 1) / kHubChunk;
@@ -753,7 +754,7 @@ fg_status run_batch_on(fg_graph *g, Workspace &ws, bool shared_ws, int grid_div,
   // partition, else one warp per query and visit; PPR is never grouped
   int Gq = 1;
   if (qtype != Q_PPR && o.mode == FG_MODE_BUFFERED)
-    Gq = o.group == 0 ? auto_group_size(g, qtype, nq, o.sched == FG_SCHED_PRIORITY && o.sched_window != 0u)
+    Gq = o.group == 0 ? auto_group_size(g, qtype, nq, o.sched == FG_SCHED_PRIORITY && o.sched_window != 0u, o.delta != 0u)
                       : o.group;
 
   if (o.mode == FG_MODE_BUFFERED && Gq > 1) {
@@ -1113,15 +1114,21 @@ namespace fg {
 // the arcs cut), SSSP with 64 queries: 4.8 and 12.7 ms one query per warp, 0.43
 // and 0.49 in groups; BFS 1.6 and 4.6 against 0.25 and 0.27 (GB300).
 bool groups_by_default(const fg_graph *g) {
-  constexpr uint32_t kRoadDegree = 64;
   constexpr int kFewPartitions = 16;
   return g->m > 0 && (2 * g->cut > g->m || (g->max_degree > kRoadDegree && g->nparts <= kFewPartitions));
 }
 
 constexpr int64_t kSmallState = 1 << 22;  // values (16 MB)
 
-int auto_group_size(const fg_graph *g, int qtype, int64_t nq, bool windowed) {
+int auto_group_size(const fg_graph *g, int qtype, int64_t nq, bool windowed, bool delayed) {
   if (!groups_by_default(g)) return 1;
+  // A window or a delta is what spares one query per warp the work that groups
+  // share: with them a small road map with a hub or two is the former's (128^2
+  // grid with a vertex of 100 arcs, 64 SSSP queries with the tuner's window: 0.89
+  // ms, 2.7 in groups; FIFO rounds 4.7 and 2.1), while from a thirtieth of the arcs at hubs
+  // on groups win up to some 32 queries and soon for all (3 %: 1 query 0.72 and 0.45, 64
+  // queries 1.17 and 2.10; 10 %: 1.24 and 0.59, 1.84 and 1.63).
+  if (qtype == Q_SSSP && (windowed || delayed) && 2 * g->cut <= g->m && 32 * g->hub_arcs < (uint64_t)g->m) return 1;
   // the widest group: fewer reads of arcs and masks for as many queries (BFS on
   // R-MAT, groups of 32 -> 64: 2^14 vertices, 64 queries 0.37 -> 0.36 ms; 2^20, 256
   // queries 5.1 -> 3.8; 2^22 20.3 -> 13.8). SSSP groups of 64 run FIFO rounds only
