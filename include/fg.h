@@ -436,6 +436,10 @@ fg_status fg_sssp_batch_noalloc(const fg_graph *g, const int32_t *src, int32_t n
  * Asynchronous on `stream`, with one exception: the first call on a graph
  * builds the graph's table of out-degrees by original id (4 * n bytes, freed
  * with the graph) and waits for it. Errors are detected on the host only.
+ * Graphs of more than 16,384 vertices take scratch from the stream-ordered
+ * allocator (80 KB + 12 * top bytes a row, up to 1,024 rows at once, and up to
+ * 10 MB for rows without a usable sample), given back by the call; with less
+ * memory fewer rows go at once, and without any the call needs none and is slower.
  */
 #define FG_NCP_MAX_TOP 4096
 fg_status fg_ncp_sweep(fg_graph *g, const float *p, int32_t nq, int32_t top, int32_t *order_out,

@@ -966,6 +966,8 @@ __global__ void __launch_bounds__(kThreads) ncp_scan_kernel(NcpArgs a) {
 // 9,000 vertices, 1 row, top 300: 44 us here and 72 through them; at the line the
 // two meet (105 rows, top 4,096: 263 us here with 16,000 vertices, 255 through
 // them with 17,000; 1 row, top 300: 57 and 70 with 17,000, top 512: 78 and 77 with 25,000).
+// It takes rows of any length and no scratch, so longer rows come here too when
+// there is no memory for the other kernels' scratch.
 constexpr int64_t kSmallRow = 1 << 14;
 constexpr size_t kSmallSmem = kInsideSmem + (size_t)kMaxTop * 4;  // and the gains
 static_assert(kSmem <= kSmallSmem, "the row is streamed in the same memory");
@@ -1104,11 +1106,7 @@ extern "C" fg_status fg_ncp_sweep(fg_graph *g, const float *p, int32_t nq, int32
   a.phi = phi_out;
   a.count = count_out;
   a.ncp = reinterpret_cast<unsigned long long *>(ncp_out);
-  const bool small = n <= kSmallRow || (n <= kSmallRow + kSmallRow / 2 && top <= 512);
-  if (a.ncp && small) {  // (else by the edge kernel)
-    ncp_profile_begin<<<(top + 255) / 256, 256, 0, stream>>>(a.ncp, top, accumulate ? 1 : 0);
-    CUDA_TRY(cudaGetLastError());
-  }
+  bool small = n <= kSmallRow || (n <= kSmallRow + kSmallRow / 2 && top <= 512);
   const bool vec = (n % 4 == 0) && aligned(p, 16);
   // Rows go through in launches of at most kRowsPerLaunch, which bounds the
   // scratch (about 80 KB + 12 * top bytes a row, from the stream-ordered
@@ -1130,8 +1128,18 @@ extern "C" fg_status fg_ncp_sweep(fg_graph *g, const float *p, int32_t nq, int32
     const cudaError_t e0 = cudaMallocAsync(reinterpret_cast<void **>(&scratch),
                                            b_hist + 4 * b_small + b_list + 3 * b_top + b_part, stream);
     if (e0 == cudaSuccess) break;
-    if (e0 != cudaErrorMemoryAllocation || rows_max == 1) CUDA_TRY(e0);
+    if (e0 != cudaErrorMemoryAllocation) CUDA_TRY(e0);
     (void)cudaGetLastError();
+    scratch = nullptr;
+    if (rows_max == 1) {  // none at all: one block a row, which streams a row of any length
+      small = true;
+      rows_max = std::min<int64_t>(nq, kRowsPerLaunch);
+      break;
+    }
+  }
+  if (a.ncp && small) {  // (else by the edge kernel)
+    ncp_profile_begin<<<(top + 255) / 256, 256, 0, stream>>>(a.ncp, top, accumulate ? 1 : 0);
+    CUDA_TRY(cudaGetLastError());
   }
   unsigned char *at = scratch;
   auto take = [&at](size_t b) {
