@@ -119,7 +119,8 @@ typedef struct {
                                half of the graph's arcs cross partitions, or it has out-degrees
                                above 64 and at most 16 partitions (but for SSSP with a
                                sched_window or a delta where such vertices have under 1/32 of
-                               the arcs), 64 (32 for SSSP with a
+                               the arcs, and on some graphs of one partition, where a
+                               query is one visit), 64 (32 for SSSP with a
                                sched_window; a smaller batch takes the smallest group that
                                holds it, and for SSSP with n * nq of at most 2^22, 8 up to 32
                                queries and 16 up to 64), else 1. PPR

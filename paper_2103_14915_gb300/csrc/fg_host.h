@@ -182,7 +182,8 @@ bool groups_by_default(const fg_graph *g);
 // of one kind: where groups_by_default, 64, or 32 for SSSP under a window, or 8
 // or 16 for SSSP with little state (the smallest of 8, 16, 32, 64 that holds a
 // smaller batch, and one that fits shared memory); else 1, as for SSSP with a
-// window or a delta on a graph of few partitions and few arcs at its hubs.
+// window or a delta on a graph of few partitions and few arcs at its hubs, and on
+// some graphs of one partition.
 int auto_group_size(const fg_graph *g, int qtype, int64_t nq, bool windowed, bool delayed);
 
 // The graph and hubs a group-engine launch of this query kind runs on.

@@ -1129,6 +1129,14 @@ int auto_group_size(const fg_graph *g, int qtype, int64_t nq, bool windowed, boo
   // on groups win up to some 32 queries and soon for all (3 %: 1 query 0.72 and 0.45, 64
   // queries 1.17 and 2.10; 10 %: 1.24 and 0.59, 1.84 and 1.63).
   if (qtype == Q_SSSP && (windowed || delayed) && 2 * g->cut <= g->m && 32 * g->hub_arcs < (uint64_t)g->m) return 1;
+  // One partition: a query is one visit that nothing waits for, and a batch takes
+  // as long as its longest visit. Groups win by what the
+  // reduced graph spares, by BFS's masks and for a handful of queries (1,024 vertices,
+  // SSSP: 25,000 arcs, 16 queries 0.97 ms and 0.76 in groups, 256 queries 1.04 and
+  // 2.09, 4,000 1.71 and 3.07; 57,000 arcs, reduced, 256 queries 2.31 and 0.59; BFS
+  // 0.37 and 0.22), but not on a few thousand arcs (200 vertices, 16 queries: SSSP
+  // 0.13 and 0.31, BFS 0.11 and 0.14).
+  if (g->nparts == 1 && (g->m < 8192 || (qtype == Q_SSSP && !g->reduced && nq > 8))) return 1;
   // the widest group: fewer reads of arcs and masks for as many queries (BFS on
   // R-MAT, groups of 32 -> 64: 2^14 vertices, 64 queries 0.37 -> 0.36 ms; 2^20, 256
   // queries 5.1 -> 3.8; 2^22 20.3 -> 13.8). SSSP groups of 64 run FIFO rounds only

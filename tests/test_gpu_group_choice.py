@@ -1,6 +1,8 @@
 """The automatic group on graphs of few partitions: a window or a delta sends
 SSSP on a road map with a lone hub to one query per warp, whose options they
-are; other batches there, and graphs whose arcs are at hubs, go to groups."""
+are; other batches there, and graphs whose arcs are at hubs, go to groups. A
+graph of one partition goes to one query per warp where neither the reduced
+graph nor BFS's masks speak for groups."""
 import numpy as np
 import pytest
 
@@ -45,5 +47,35 @@ def test_choice(graph):
             st, stats = fg.fg_stats(h)
             fg.check(st)
             assert (stats.group == 1) == (alone and graph == "road"), (opts, stats.group)
+    finally:
+        fg.fg_graph_destroy(h)
+
+
+@pytest.mark.parametrize("n,edges,groups", [(200, 1200, (False, False)), (1000, 9000, (False, True)),
+                                            (1000, 40000, (True, True))])
+def test_one_partition(n, edges, groups):
+    """groups: of SSSP, BFS; the densest graph has a reduced one."""
+    r = np.random.RandomState(n)
+    u, v = (n * r.rand(edges) ** 3).astype(np.int64), r.randint(0, n, edges)
+    u, v, w = np.r_[u, v], np.r_[v, u], np.tile(r.randint(1, 256, edges), 2)
+    order = np.argsort(u, kind="stable")
+    rp = np.zeros(n + 1, np.int64)
+    rp[1:] = np.cumsum(np.bincount(u, minlength=n))
+    g = inputs.Graph(n, rp, v[order].astype(np.int32), w[order].astype(np.int32), True)
+    assert g.out_degree().max() > 64
+    srcs = np.resize(np.arange(n), 300).astype(np.int32)
+    st, h = fg.fg_graph_create(g.n, g.m, g.row_ptr, g.col, g.w, 0)
+    fg.check(st)
+    s_d = torch.from_numpy(srcs).to(DEV)
+    out = torch.empty((len(srcs), g.n), dtype=torch.int32, device=DEV)
+    try:
+        for call, ref, grouped in ((fg.fg_sssp_batch, oracle.sssp(g, srcs), groups[0]),
+                                   (fg.fg_bfs_batch, oracle.bfs(g, srcs), groups[1])):
+            fg.check(call(h, s_d, len(srcs), out))
+            fg.check(fg.fg_sync())
+            assert np.array_equal(out.cpu().numpy().view(np.uint32), ref)
+            st, stats = fg.fg_stats(h)
+            fg.check(st)
+            assert (stats.group > 1) == grouped
     finally:
         fg.fg_graph_destroy(h)
