@@ -37,7 +37,8 @@
 // much again of degrees from L2), order 55, inside 100, scan 18, and 0.33 ms for
 // the call. One block per row doing all of it took 1.94 ms: 105 blocks leave a
 // third of the SMs idle, and the threshold that its buffer finds on the way lets
-// five times as many keys in. Rows of few vertices take one block (below).
+// five times as many keys in. Rows of few vertices take one
+// block, and few rows with a small `top` two kernels (below).
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
@@ -708,7 +709,7 @@ constexpr int kStreamParts = 16;
 constexpr int64_t kStreamSlots = 128;
 
 __device__ __forceinline__ bool list_usable(const NcpArgs &a, int64_t row) {
-  return a.listed[row] <= (uint32_t)kCap && a.listed[row] >= min((uint32_t)a.top, a.positive[row]);
+  return a.list != nullptr && a.listed[row] <= (uint32_t)kCap && a.listed[row] >= min((uint32_t)a.top, a.positive[row]);
 }
 
 struct RowStream {
@@ -969,10 +970,22 @@ __global__ void __launch_bounds__(kThreads) ncp_scan_kernel(NcpArgs a) {
 // It takes rows of any length and no scratch, so longer rows come here too when
 // there is no memory for the other kernels' scratch.
 constexpr int64_t kSmallRow = 1 << 14;
+// Little work and a small `top` are launches mostly, too: there the stream kernel's
+// blocks leave a row's keys by parts and this kernel merges them, two launches for the
+// six that find and filter a list. Calls back to back, top 16 / 64 / 256: 4 rows of 2^15
+// vertices 33 / 36 / 51 us, and 50 / 52 / 60 by lists; 8 rows of 2^17 43 / 47 / 61 and 56 / 59 /
+// 63; 2^18 56 / 59 / 76 and 60 / 62 / 68; 1 row of 2^20 85 / 94 / 113 and 60 / 58 / 64; top
+// 512, 2^16 vertices 74 and 68.
+constexpr int64_t kFewRow = 1 << 18;
+constexpr int32_t kFewTop = 256;
+constexpr int64_t kFewRowTop = 1 << 25;  // vertices of a row * top
+constexpr int64_t kFewElems = 1 << 21;   // of the call
+static_assert(kFewElems / kSmallRow <= kStreamSlots, "the stream kernel has room for every row of such a call");
 constexpr size_t kSmallSmem = kInsideSmem + (size_t)kMaxTop * 4;  // and the gains
 static_assert(kSmem <= kSmallSmem, "the row is streamed in the same memory");
 
-__global__ void __launch_bounds__(kThreads) ncp_small_kernel(NcpArgs a, bool vec) {
+// parts > 1: the row's keys come from the stream kernel's blocks
+__global__ void __launch_bounds__(kThreads) ncp_small_kernel(NcpArgs a, bool vec, int parts) {
   extern __shared__ __align__(16) unsigned char smem[];
   unsigned long long *cand = reinterpret_cast<unsigned long long *>(smem);
   __shared__ RowStream rs;
@@ -980,7 +993,10 @@ __global__ void __launch_bounds__(kThreads) ncp_small_kernel(NcpArgs a, bool vec
   const int64_t row = blockIdx.x;
   const Stream st = rs.on(smem);
   stream_begin(st);
-  stream_part(a, row, vec, st, 0, 1);
+  if (parts > 1)
+    stream_keys(a.part + (size_t)row * parts * (size_t)a.top, (int64_t)parts * a.top, st, (uint32_t)a.top);
+  else
+    stream_part(a, row, vec, st, 0, 1);
   const uint32_t L = min(*st.n_buf, (uint32_t)a.top);
   sort_keys(cand, L);
   // the sorted keys take the first kMaxTop * 8 bytes, hash keys later; the
@@ -1114,17 +1130,19 @@ extern "C" fg_status fg_ncp_sweep(fg_graph *g, const float *p, int32_t nq, int32
   constexpr int64_t kRowsPerLaunch = 1024;
   auto up = [](size_t b) { return (b + 255) / 256 * 256; };
   int64_t rows_max = std::min<int64_t>(nq, kRowsPerLaunch);
+  bool few = !small && n <= kFewRow && top <= kFewTop && n * top <= kFewRowTop && n * nq <= kFewElems;
   size_t b_hist = 0, b_small = 0, b_list = 0, b_top = 0, b_part = 0;
   int stream_parts = 0;
   unsigned char *scratch = nullptr;
   for (; !small; rows_max = (rows_max + 1) / 2) {  // fewer rows a launch where memory is short
-    b_hist = up((size_t)rows_max * kBins * 4);
+    b_hist = up((size_t)rows_max * kBins * 4);  // (few: only the parts)
     b_small = up((size_t)rows_max * 4);
     b_list = up((size_t)rows_max * kCap * 8);
     b_top = up((size_t)rows_max * ((size_t)top + 1) * 4);
     // two blocks an SM; one part (in the order kernel) for rows that one block streams in 50 us
-    stream_parts = n <= kSampleAll ? 1 : (int)std::max<int64_t>(1, std::min<int64_t>(kStreamParts, 304 / rows_max));
+    stream_parts = n <= kSampleAll && !few ? 1 : (int)std::max<int64_t>(1, std::min<int64_t>(kStreamParts, 304 / rows_max));
     b_part = stream_parts == 1 ? 0 : up((size_t)std::min(rows_max, kStreamSlots) * (size_t)stream_parts * (size_t)top * 8);
+    if (few) b_hist = b_small = b_list = b_top = 0;
     const cudaError_t e0 = cudaMallocAsync(reinterpret_cast<void **>(&scratch),
                                            b_hist + 4 * b_small + b_list + 3 * b_top + b_part, stream);
     if (e0 == cudaSuccess) break;
@@ -1133,11 +1151,12 @@ extern "C" fg_status fg_ncp_sweep(fg_graph *g, const float *p, int32_t nq, int32
     scratch = nullptr;
     if (rows_max == 1) {  // none at all: one block a row, which streams a row of any length
       small = true;
+      few = false;
       rows_max = std::min<int64_t>(nq, kRowsPerLaunch);
       break;
     }
   }
-  if (a.ncp && small) {  // (else by the edge kernel)
+  if (a.ncp && (small || few)) {  // (else by the edge kernel)
     ncp_profile_begin<<<(top + 255) / 256, 256, 0, stream>>>(a.ncp, top, accumulate ? 1 : 0);
     CUDA_TRY(cudaGetLastError());
   }
@@ -1153,7 +1172,7 @@ extern "C" fg_status fg_ncp_sweep(fg_graph *g, const float *p, int32_t nq, int32
   a.hist = reinterpret_cast<uint32_t *>(take(b_hist));
   a.edge = reinterpret_cast<uint32_t *>(take(b_small));
   a.kept = reinterpret_cast<uint32_t *>(take(b_small));
-  a.list = reinterpret_cast<unsigned long long *>(take(b_list));
+  a.list = few ? nullptr : reinterpret_cast<unsigned long long *>(take(b_list));
   a.ids = reinterpret_cast<uint32_t *>(take(b_top));
   a.gain = reinterpret_cast<int32_t *>(take(b_top));
   a.first = reinterpret_cast<uint32_t *>(take(b_top));
@@ -1174,8 +1193,10 @@ extern "C" fg_status fg_ncp_sweep(fg_graph *g, const float *p, int32_t nq, int32
     if (a.order) b.order = a.order + r0 * top;
     if (a.phi) b.phi = a.phi + r0 * top;
     if (a.count) b.count = a.count + r0;
-    if (small) {
-      ncp_small_kernel<<<rows, kThreads, kSmallSmem, stream>>>(b, vec);
+    if (small || few) {
+      if (few && stream_parts > 1)
+        ncp_stream_kernel<<<rows * stream_parts, kThreads, kSmem, stream>>>(b, vec, stream_parts);
+      ncp_small_kernel<<<rows, kThreads, kSmallSmem, stream>>>(b, vec, few ? stream_parts : 1);
       e = cudaGetLastError();
       continue;
     }
