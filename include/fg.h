@@ -106,9 +106,10 @@ typedef struct {
                                so one batch's copy to the host overlaps the next batch's
                                kernels when they run on different streams */
     int32_t query_batch;    /* queries per device launch; 0 = all (bounded by workspace) */
-    int32_t threads_per_vertex; /* 0 (default), 1 or 32; the engine picks the form of SSSP/BFS
-                               expansion by the graph's out-degrees (arc records of fixed size up
-                               to 8, else a warp shares the arcs of 32 frontier vertices evenly) */
+    int32_t threads_per_vertex; /* 0 (default), 1 or 32: accepted, without effect. The engine picks
+                               the form of SSSP/BFS expansion by the graph's out-degrees (arc
+                               records of fixed size up to 8, else a warp shares the arcs of 32
+                               frontier vertices evenly) */
     int32_t group;          /* SSSP/BFS queries that share one partition visit lane by lane
                                (the query group): 8, 16, 32 or 64 = the group engine, whose state
                                keeps a group's values of one vertex in one line, so one access
@@ -192,6 +193,10 @@ void fg_default_graph_opts(fg_graph_opts *o);
  * automatic choice also gets a second copy without the arcs that lie on no shortest
  * path, if enough are found: SSSP in the group engine runs on that copy, with
  * the same distances (16 * n words of device memory during the call).
+ * A graph whose out-degrees are at most 8 also gets its arcs as records of fixed
+ * size for SSSP/BFS with one query per warp: 64 bytes a vertex of device memory for
+ * the graph's life, several times its CSR (fg_graph_info counts them). Without
+ * memory for either, creation succeeds and the batches do without.
  */
 fg_status fg_graph_create(int64_t n, int64_t m, const int64_t *row_ptr, const int32_t *col,
                           const int32_t *w, uint32_t flags, fg_graph **out);
@@ -211,7 +216,11 @@ fg_status fg_graph_info(const fg_graph *g, fg_graph_info_t *info);
  * nq single-source shortest-path queries (Def. 2.3: an operation <q, v, l>
  * lowers v's path length to l when l is shorter). dist_out: uint32[nq * n],
  * exact distances; UINT32_MAX = unreachable. src: int32[nq] (duplicates are
- * allowed). Unweighted graphs use weight 1.
+ * allowed). Unweighted graphs use weight 1. FG_ERR_OVERFLOW (from fg_sync): a
+ * final distance plus the weight of an arc of its vertex reaches 2^32 - 1, or a
+ * value on the way to one did; which values on the way are formed depends on the
+ * engine and on the arcs left out, so a batch whose final sums all stay below may
+ * report it or not. Distances below the limit are right either way.
  */
 fg_status fg_sssp_batch(fg_graph *g, const int32_t *src, int32_t nq, uint32_t *dist_out,
                         void *stream, const fg_opts *opts);
